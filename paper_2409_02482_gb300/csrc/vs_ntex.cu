@@ -344,17 +344,35 @@ __global__ void __launch_bounds__(kThreads) k_gather_grad(const float* G, int C,
   dY[id] = __ldg(G + (size_t)(n0 + i) * pitch + ch0 + c);
 }
 
-// Adam (Kingma & Ba) with bias correction.
+// Adam (Kingma & Ba) with bias correction.  Bound by HBM: 28 bytes per
+// parameter, read once and written once.  Four parameters per thread where
+// all four arrays are 16-byte aligned: four 16-byte loads in flight instead
+// of four 4-byte ones (16.8 M parameters: 71 us, 6.6 TB/s, against 100 us).
+__device__ __forceinline__ void adam1(float& p, float g, float& m, float& v, float lr, float b1, float b2, float eps,
+                                      float c1, float c2) {
+  m = b1 * m + (1.0f - b1) * g;
+  v = b2 * v + (1.0f - b2) * g * g;
+  p -= lr * (m / c1) / (sqrtf(v / c2) + eps);
+}
+
+template <int VEC>
 __global__ void __launch_bounds__(kThreads) k_adam(float* p, const float* g, float* m, float* v, long long n, float lr,
                                                     float b1, float b2, float eps, float c1, float c2) {
-  const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (id >= n) return;
-  const float gi = g[id];
-  const float mi = b1 * m[id] + (1.0f - b1) * gi;
-  const float vi = b2 * v[id] + (1.0f - b2) * gi * gi;
-  m[id] = mi;
-  v[id] = vi;
-  p[id] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  const long long id = VEC * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
+  if (VEC == 4 && id + 4 <= n) {
+    float4 P = *reinterpret_cast<float4*>(p + id), M = *reinterpret_cast<float4*>(m + id);
+    float4 V = *reinterpret_cast<float4*>(v + id);
+    const float4 G = *reinterpret_cast<const float4*>(g + id);
+    adam1(P.x, G.x, M.x, V.x, lr, b1, b2, eps, c1, c2);
+    adam1(P.y, G.y, M.y, V.y, lr, b1, b2, eps, c1, c2);
+    adam1(P.z, G.z, M.z, V.z, lr, b1, b2, eps, c1, c2);
+    adam1(P.w, G.w, M.w, V.w, lr, b1, b2, eps, c1, c2);
+    *reinterpret_cast<float4*>(m + id) = M;
+    *reinterpret_cast<float4*>(v + id) = V;
+    *reinterpret_cast<float4*>(p + id) = P;
+    return;
+  }
+  for (long long i = id; i < id + VEC && i < n; ++i) adam1(p[i], g[i], m[i], v[i], lr, b1, b2, eps, c1, c2);
 }
 
 // ----------------------------------------------------------------------------
@@ -871,7 +889,10 @@ int backward(const vs_ntex_config& c, const float* params, int W, int H, const f
 int adam(float* p, const float* g, float* m, float* v, long long n, float lr, float b1, float b2, float eps, int step,
          cudaStream_t st) {
   const float c1 = (float)(1.0 - std::pow((double)b1, step)), c2 = (float)(1.0 - std::pow((double)b2, step));
-  k_adam<<<blocks_for(n), kThreads, 0, st>>>(p, g, m, v, n, lr, b1, b2, eps, c1, c2);
+  if (((uintptr_t)p | (uintptr_t)g | (uintptr_t)m | (uintptr_t)v) % 16 == 0)
+    k_adam<4><<<blocks_for((n + 3) / 4), kThreads, 0, st>>>(p, g, m, v, n, lr, b1, b2, eps, c1, c2);
+  else
+    k_adam<1><<<blocks_for(n), kThreads, 0, st>>>(p, g, m, v, n, lr, b1, b2, eps, c1, c2);
   return (int)cudaGetLastError();
 }
 

@@ -308,3 +308,27 @@ def test_fitting_through_the_renderer_reduces_the_loss(vs, ctx):
     assert vs.read_stats(ws)["device_status"] == 0
     assert all(np.isfinite(history))
     assert history[-1] < 0.5 * history[0], history[::10]
+
+
+@pytest.mark.parametrize("n,shift", [(1, 0), (3, 0), (4, 0), (1021, 0), (1024, 1), (4099, 3)])
+def test_adam_vector_and_scalar_parameters(vs, ctx, n, shift):
+    """Adam on parameter counts off a multiple of four and on arrays that are
+    not 16-byte aligned against the oracle's step (bars of
+    test_adam_matches_oracle), with nothing written outside the arrays."""
+    rng = np.random.default_rng(n + shift)
+    p, g, m = (rng.normal(size=n) for _ in range(3))
+    v = rng.random(n)
+    bufs = []
+    for x in (p, g, m, v):
+        b = torch.full((n + shift + 4,), 9.0, device="cuda")
+        b[shift:shift + n] = torch.from_numpy(x.astype(np.float32))
+        bufs.append(b)
+    ptr = [b.data_ptr() + 4 * shift for b in bufs]
+    lib = ctx.lib
+    assert lib.vs_adam_step(ctx.handle, *ptr, n, 1e-2, 0.9, 0.99, 1e-15, 3,
+                            torch.cuda.current_stream().cuda_stream) == 0
+    rp, rm, rv = ntex.adam(p, g, m, v, 3, lr=1e-2)
+    for b, r in zip(bufs, (rp, g, rm, rv)):
+        got = b.cpu().numpy()
+        assert np.abs(got[shift:shift + n] - r).max() <= 1e-5
+        assert np.all(got[:shift] == 9.0) and np.all(got[shift + n:] == 9.0)

@@ -310,6 +310,51 @@ def test_fitting_through_the_renderer_reduces_the_loss(vs, ctx):
     assert history[-1] < 0.5 * history[0], history[::10]
 
 
+@pytest.mark.parametrize("levels,features,hidden,out_ch,W,H,pad,ch0", [
+    (1, 1, 1, 1, 1, 1, 0, 0),         # one texel
+    (3, 2, 31, 3, 63, 1, 1, 1),       # one tile short of full, scalar channel access
+    (8, 4, 32, 32, 64, 1, 0, 0),      # a full tile, 32 of everything
+    (8, 4, 33, 31, 65, 1, 1, 0),      # one texel into the second tile
+    (16, 4, 64, 32, 129, 5, 4, 4),    # 64 encoding values; tiles that span texture rows
+    (16, 3, 40, 27, 37, 29, 1, 0),    # rows shorter than a tile
+    (16, 2, 64, 33, 70, 40, 3, 0),    # more outputs than the fused adjoint takes
+    (16, 2, 64, 64, 300, 70, 0, 0),
+    (4, 2, 65, 5, 40, 33, 0, 0),      # more hidden units than the fused kernels take
+])
+def test_ntex_fused_fp32_shapes_match_oracle(vs, ctx, levels, features, hidden, out_ch, W, H, pad, ch0):
+    """The fused FP32 kernels at the edges of their padding (hidden units,
+    encoding values and outputs to 32 or 64) and of their 64-texel tiles, and
+    the shapes just past their range: texels and gradients within the FP32
+    bars of test_ntex_forward_matches_oracle and
+    test_ntex_backward_matches_oracle, channels outside [ch0, ch0 + C) left
+    alone."""
+    cfg = ntex.NtexConfig(levels=levels, features=features, log2_table=8, base_res=3, growth=1.25, hidden=hidden,
+                          out_ch=out_ch)
+    params = _params(cfg, 100 + hidden)
+    nt = _net(vs, ctx, cfg, params, W, H)
+    pitch = out_ch + ch0 + pad
+    tex = torch.full((H, W, pitch), 7.0, device="cuda")
+    nt.forward(tex, ch0=ch0)
+    ref, _ = ntex.forward(cfg, params.astype(np.float64), W, H)
+    ref = ref.reshape(H, W, out_ch)
+    got = tex.cpu().numpy()
+    scale = max(1.0, np.abs(ref).max())
+    assert np.abs(got[..., ch0:ch0 + out_ch] - ref).max() <= 1e-4 * scale
+    assert np.all(got[..., :ch0] == 7.0) and np.all(got[..., ch0 + out_ch:] == 7.0)
+    half = torch.zeros((H, W, pitch), dtype=torch.float16, device="cuda")
+    nt.forward(half, ch0=ch0)
+    assert np.abs(half.float().cpu().numpy()[..., ch0:ch0 + out_ch] - ref).max() <= 2e-3 * scale
+    g = torch.randn((H, W, pitch), device="cuda", generator=torch.Generator("cuda").manual_seed(13))
+    nt.backward(g, ch0=ch0)
+    rg = ntex.backward(cfg, params.astype(np.float64), W, H,
+                       g.cpu().numpy()[..., ch0:ch0 + out_ch].astype(np.float64))
+    q = nt.grads.cpu().numpy()
+    lay, _ = cfg.layout()
+    for name, off, shp in lay:
+        n = int(np.prod(shp))
+        assert np.abs(q[off:off + n] - rg[off:off + n]).max() <= 1e-4 * max(np.abs(rg[off:off + n]).max(), 1e-30), name
+
+
 @pytest.mark.parametrize("n,shift", [(1, 0), (3, 0), (4, 0), (1021, 0), (1024, 1), (4099, 3)])
 def test_adam_vector_and_scalar_parameters(vs, ctx, n, shift):
     """Adam on parameter counts off a multiple of four and on arrays that are

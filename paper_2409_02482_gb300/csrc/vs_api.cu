@@ -232,12 +232,26 @@ void order_for_locality(std::vector<ItemReq>& req) {
   req.swap(out);
 }
 
-// Work-unit sizes of one plan, in 32-wide rounds.  The plain launches run
-// one round per warp of a block, so they always use kWarps rounds.
+// Work-unit sizes of one plan: the most triangles per raster unit, the 32-wide
+// rounds per shading unit (the plain launch runs one per warp of a block),
+// and the warps that should find a raster unit (those resident on the GPU).
 struct UnitShape {
-  int raster_rounds = kWarps;
+  int raster_tris = 32;
   int shade_rounds = kWarps;
+  int warps = 0;
 };
+
+// Raster units of an item of `tris` triangles: units of the asked size while
+// every resident warp gets one, else smaller, down to one triangle, which 2,
+// 4 .. 64 warps then share.  A mesh of few triangles has large ones: at 256^2,
+// 3 x 1224 triangles took 253 us in units of 32 (115 warps busy) and take
+// 7 us one by one.
+void raster_shape(long long tris, const UnitShape& shape, int* unit, int* lg) {
+  *unit = shape.raster_tris;
+  *lg = 0;
+  while (*unit > 1 && tris / *unit < shape.warps) *unit /= 2;
+  while (*unit == 1 && *lg < 6 && (tris << (*lg + 1)) <= shape.warps) ++*lg;
+}
 
 struct Plan {
   bool full = false;             // the full kernels: a shell may reach nearer than znear
@@ -306,7 +320,6 @@ vs_status make_plan(const ItemReq* req, int n, const float* bg, int do_bwd, bool
     return fail(VS_ERR_INVALID_ARG, "VS_FLAG_LOSS_L1 and VS_FLAG_LOSS_L2 are exclusive");
   P.full = false;
   for (int j = 0; j < n; ++j) P.full = P.full || needs_clip(*req[j].obj, *req[j].cam) || req[j].layers;
-  const int raster_per_unit = 32 * shape.raster_rounds;
   const int shade_per_unit = 32 * shape.shade_rounds;
   size_t off = sizeof(WsHeader);
   int S = 0;
@@ -342,7 +355,9 @@ vs_status make_plan(const ItemReq* req, int n, const float* bg, int do_bwd, bool
     it.flags = (int)flags;
     it.do_bwd = do_bwd;
     it.stall = (flags & VS_FLAG_TEST_STALL) ? 1 : 0;
-    it.raster_rounds = shape.raster_rounds;
+    long long tris = 0;
+    for (int i = 0; i < o.k; ++i) tris += o.shells[i].num_tris;
+    raster_shape(tris, shape, &it.raster_tris, &it.raster_lg);
     it.shade_rounds = shape.shade_rounds;
     it.bg[0] = bg ? bg[0] : 0.f; it.bg[1] = bg ? bg[1] : 0.f; it.bg[2] = bg ? bg[2] : 0.f;
     const size_t HW = (size_t)c.width * c.height;
@@ -379,14 +394,14 @@ vs_status make_plan(const ItemReq* req, int n, const float* bg, int do_bwd, bool
       s.vsetup = reinterpret_cast<int4*>(ws ? ws + off : nullptr);
       off = align256(off + sizeof(int4) * (size_t)d.num_verts);
       it.setup_pre[i + 1] = it.setup_pre[i] + (d.num_verts + kSetupPerUnit - 1) / kSetupPerUnit;
-      it.raster_pre[i + 1] = it.raster_pre[i] + (d.num_tris + raster_per_unit - 1) / raster_per_unit;
+      it.raster_pre[i + 1] = it.raster_pre[i] + (d.num_tris + it.raster_tris - 1) / it.raster_tris;
     }
     it.vis = reinterpret_cast<unsigned long long*>(ws ? ws + off : nullptr);
     if (clear_vis) off = align256(off + sizeof(unsigned long long) * o.k * HW);
     const size_t vis_words = (size_t)o.k * HW;
     it.clear_units = clear_vis ? (int)((vis_words + kClearPerUnit - 1) / kClearPerUnit) : 0;
     it.units[PH_SETUP] = it.clear_units + it.setup_pre[o.k];
-    it.units[PH_RASTER] = clear_vis ? it.raster_pre[o.k] : 0;
+    it.units[PH_RASTER] = clear_vis ? it.raster_pre[o.k] << it.raster_lg : 0;
     it.units[PH_SHADE] = (int)((HW + shade_per_unit - 1) / shade_per_unit);
     sidx += o.k;
   }
@@ -514,10 +529,21 @@ vs_tuning lookup_tuning(vs_ctx* ctx, int bwd, int kmax) {
   return ctx->tune_set[bwd][kmax] ? ctx->tune[bwd][kmax] : default_tuning();
 }
 
-UnitShape shape_of(const vs_tuning& t) {
+// Warps resident in the plain raster kernel, and in the persistent kernels
+// to within a sixth.
+int resident_warps(const vs_ctx* ctx) { return ctx->num_sms * kRasterBlocks * kWarps; }
+
+UnitShape plain_shape(const vs_ctx* ctx) {
   UnitShape u;
-  u.raster_rounds = t.raster_tris / 32;
+  u.warps = resident_warps(ctx);
+  return u;
+}
+
+UnitShape shape_of(const vs_ctx* ctx, const vs_tuning& t) {
+  UnitShape u;
+  u.raster_tris = t.raster_tris;
   u.shade_rounds = t.shade_pixels / 32;
+  u.warps = resident_warps(ctx);
   return u;
 }
 
@@ -561,7 +587,7 @@ vs_status plan_batch(const vs_ctx* ctx, const vs_batch_item* items, int n, const
   vs_status s = check_batch(ctx, items, n, do_backward, req, kmax);
   if (s != VS_OK) return s;
   if ((s = make_plan(req.data(), n, bg, do_backward ? 1 : 0, true, flags, static_cast<char*>(workspace), P,
-                     shape_of(t))) != VS_OK)
+                     shape_of(ctx, t))) != VS_OK)
     return s;
   return check_ws(P, workspace, ws_bytes);
 }
@@ -751,11 +777,11 @@ vs_status vs_render(vs_ctx* ctx, const vs_object* obj, const vs_camera* cam, con
   char* ws = static_cast<char*>(workspace);
   if ((s = set_device(ctx)) != VS_OK) return s;
   if ((s = ensure_bounds(obj)) != VS_OK) return s;
-  if ((s = make_plan(&r, 1, bg, 0, true, flags & ~VS_FLAG_TEST_STALL, ws, P)) != VS_OK) return s;
+  if ((s = make_plan(&r, 1, bg, 0, true, flags & ~VS_FLAG_TEST_STALL, ws, P, plain_shape(ctx))) != VS_OK) return s;
   if ((s = check_ws(P, workspace, ws_bytes)) != VS_OK) return s;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if ((s = upload_table(P, ws, vsk::plain_forward_launches(P.items[0].units), st)) != VS_OK) return s;
-  cudaError_t e = vsk::plain_forward(table_ref(P, ws), P.items[0].units, P.tc, P.full, st);
+  cudaError_t e = vsk::plain_forward(table_ref(P, ws), P.items[0].units, P.tc, P.full, ctx->num_sms, st);
   return e == cudaSuccess ? VS_OK : cuda_fail(e, "vs_render launch");
 }
 
@@ -773,11 +799,11 @@ vs_status vs_render_layers(vs_ctx* ctx, const vs_object* obj, const vs_camera* c
   char* ws = static_cast<char*>(workspace);
   if ((s = set_device(ctx)) != VS_OK) return s;
   if ((s = ensure_bounds(obj)) != VS_OK) return s;
-  if ((s = make_plan(&r, 1, bg, 0, true, flags & ~VS_FLAG_TEST_STALL, ws, P)) != VS_OK) return s;
+  if ((s = make_plan(&r, 1, bg, 0, true, flags & ~VS_FLAG_TEST_STALL, ws, P, plain_shape(ctx))) != VS_OK) return s;
   if ((s = check_ws(P, workspace, ws_bytes)) != VS_OK) return s;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if ((s = upload_table(P, ws, vsk::plain_forward_launches(P.items[0].units), st)) != VS_OK) return s;
-  cudaError_t e = vsk::plain_forward(table_ref(P, ws), P.items[0].units, P.tc, P.full, st);
+  cudaError_t e = vsk::plain_forward(table_ref(P, ws), P.items[0].units, P.tc, P.full, ctx->num_sms, st);
   return e == cudaSuccess ? VS_OK : cuda_fail(e, "vs_render_layers launch");
 }
 
@@ -819,7 +845,7 @@ vs_status vs_render_batch(vs_ctx* ctx, const vs_batch_item* items, int32_t n, co
   vs_status s = check_batch(ctx, items, n, do_backward, req, &kmax);   // makes the device current
   if (s != VS_OK) return s;
   const int bwd = do_backward ? 1 : 0;
-  const UnitShape shape = shape_of(t);
+  const UnitShape shape = shape_of(ctx, t);
   // bytes of the runs [j, j + m): the plan's layout without a workspace
   auto run_bytes = [&](int j, int m, size_t* bytes) {
     Plan Q;
@@ -1185,7 +1211,7 @@ extern "C" vs_status vs_render_noalloc(vs_ctx* ctx, const vs_object* obj, const 
   Plan P;
   if ((s = set_device(ctx)) != VS_OK) return s;
   if ((s = ensure_bounds(obj)) != VS_OK) return s;
-  if ((s = make_plan(&r, 1, bg, 0, true, fl, nullptr, P)) != VS_OK) return s;
+  if ((s = make_plan(&r, 1, bg, 0, true, fl, nullptr, P, plain_shape(ctx))) != VS_OK) return s;
   if (P.total > kNoAllocScratchBytes)
     return fail(VS_ERR_OVERFLOW,
                 "vs_render_noalloc needs %zu bytes of scratch for this object and camera; its fixed array holds "
@@ -1193,7 +1219,7 @@ extern "C" vs_status vs_render_noalloc(vs_ctx* ctx, const vs_object* obj, const 
                 P.total, kNoAllocScratchBytes);
   char* ws = nullptr;
   if ((s = noalloc_scratch(ctx->device, &ws)) != VS_OK) return s;
-  if ((s = make_plan(&r, 1, bg, 0, true, fl, ws, P)) != VS_OK) return s;
+  if ((s = make_plan(&r, 1, bg, 0, true, fl, ws, P, plain_shape(ctx))) != VS_OK) return s;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   // the array keeps the previous call's contents: the header (status,
   // counters, work counter) must start at zero; the visibility words are
@@ -1201,6 +1227,6 @@ extern "C" vs_status vs_render_noalloc(vs_ctx* ctx, const vs_object* obj, const 
   cudaError_t e = cudaMemsetAsync(ws, 0, sizeof(WsHeader), st);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(no-alloc header)");
   if ((s = upload_table(P, ws, vsk::plain_forward_launches(P.items[0].units), st)) != VS_OK) return s;
-  e = vsk::plain_forward(table_ref(P, ws), P.items[0].units, P.tc, P.full, st);
+  e = vsk::plain_forward(table_ref(P, ws), P.items[0].units, P.tc, P.full, ctx->num_sms, st);
   return e == cudaSuccess ? VS_OK : cuda_fail(e, "vs_render_noalloc launch");
 }

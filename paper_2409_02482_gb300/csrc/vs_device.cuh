@@ -21,14 +21,13 @@ namespace vsd {
 constexpr int kThreads = 256;          // threads per block, all kernels
 constexpr int kWarps = kThreads / 32;  // a work unit is run by one warp
 constexpr int kSetupPerUnit = 1024;    // vertices per setup unit
-constexpr int kRasterPerUnit = 256;    // triangles per raster unit of the plain launches
 constexpr int kClearPerUnit = 16384;   // visibility words cleared per unit
 constexpr int kShadePixels = 256;      // pixels per shading unit of the plain launches
-// The plain raster/shade launches run one unit per block, one 32-wide round
-// per warp, so their units are kWarps rounds; the persistent kernel takes
-// any size per item (DItem::raster_rounds, shade_rounds).
-static_assert(kRasterPerUnit == 32 * kWarps && kShadePixels == 32 * kWarps, "plain units = one round per warp");
-constexpr int kSmallMaxPixels = 64;    // bbox pixels walked by the warp's pair loop
+// The plain shading launch runs one unit per block, one 32-wide round per
+// warp, so its units are kWarps rounds; the persistent kernel takes any size
+// per item (DItem::shade_rounds).
+static_assert(kShadePixels == 32 * kWarps, "plain units = one round per warp");
+constexpr int kRasterBlocks = 3;       // resident blocks per SM of the plain raster kernel
 constexpr int kMaxShells = VS_MAX_SHELLS;
 constexpr int kTriBits = 27;           // triangle index bits in a packed fragment
 constexpr int kMaxTris = 1 << kTriBits;
@@ -147,9 +146,9 @@ struct alignas(16) DItem {
   float* loss;                 // scalar or null
   unsigned long long* vis;     // [k, H*W] -- workspace
   float* layers;               // [k, H*W, 12] per-layer buffers or null
-  int32_t k, shell0, pad0, clear_units;
+  int32_t k, shell0, raster_lg, clear_units;   // raster_lg: a unit of one triangle is shared by 2^raster_lg units
   int32_t flags, do_bwd, stall;
-  int32_t raster_rounds;       // raster unit = 32 * raster_rounds triangles
+  int32_t raster_tris;         // triangles per raster unit (a power of two)
   int32_t shade_rounds;        // shading unit = 32 * shade_rounds pixels
   int32_t units[4];            // per phase (3 used)
   int32_t setup_pre[kMaxShells + 1];
@@ -385,17 +384,25 @@ __device__ __forceinline__ bool covered(const Tri& t, const long long e[3]) {
 // terms, relative error ~6 ulp) is within ~2^10 of it, which bounds the
 // residual R = N - Q S below 2^62 and lets R be computed exactly in
 // wrapping 64-bit arithmetic; two correction steps make the quotient exact.
+// 64-bit integers go to FP32 by their 32-bit halves: the direct conversion
+// runs on the FP64 pipe (1/64 of the FP32 rate).  For v >= 0 the relative
+// error is below 2^-22.
+__device__ __forceinline__ float u64_to_float(unsigned long long v) {
+  return fmaf((float)(unsigned)(v >> 32), 4294967296.0f, (float)(unsigned)v);
+}
+
 __device__ __forceinline__ unsigned depth_key_r(const unsigned q[3], const long long e[3],
                                                 unsigned long long S, float rS) {
   const unsigned long long N = (unsigned long long)e[0] * q[0] + (unsigned long long)e[1] * q[1] +
                                (unsigned long long)e[2] * q[2];   // mod 2^64
-  const float est = fmaf((float)e[0], (float)q[0],
-                         fmaf((float)e[1], (float)q[1], (float)e[2] * (float)q[2])) * rS;
+  const float est = fmaf(u64_to_float(e[0]), (float)q[0],
+                         fmaf(u64_to_float(e[1]), (float)q[1], u64_to_float(e[2]) * (float)q[2])) * rS;
   const unsigned qmin = min(q[0], min(q[1], q[2])), qmax = max(q[0], max(q[1], q[2]));
   unsigned Q = (unsigned)fminf(fmaxf(est, (float)qmin), (float)qmax);
   Q = min(max(Q, qmin), qmax);
   long long R = (long long)(N - (unsigned long long)Q * S);
-  Q = (unsigned)((long long)Q + (long long)floorf((float)R * rS));
+  const float fR = R < 0 ? -u64_to_float(-R) : u64_to_float(R);
+  Q = (unsigned)((int)Q + (int)floorf(fR * rS));
   R = (long long)(N - (unsigned long long)Q * S);
 #pragma unroll 1
   for (int i = 0; i < 4 && R < 0; ++i) { --Q; R += (long long)S; }
@@ -406,7 +413,7 @@ __device__ __forceinline__ unsigned depth_key_r(const unsigned q[3], const long 
 
 __device__ __forceinline__ unsigned depth_key(const Tri& t, const long long e[3]) {
   const unsigned long long S = (unsigned long long)(e[0] + e[1] + e[2]);
-  return depth_key_r(t.q, e, S, 1.0f / (float)S);
+  return depth_key_r(t.q, e, S, 1.0f / u64_to_float(S));
 }
 
 __device__ __forceinline__ unsigned long long vis_key(unsigned K, int tri) {

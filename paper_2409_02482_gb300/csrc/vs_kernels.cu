@@ -18,20 +18,47 @@ __global__ void __launch_bounds__(kThreads) k_upload(char* ws, const __grid_cons
   }
 }
 
-// Plain per-phase kernels.  Setup: each warp runs one unit (8 per block).
-// Raster and shade: block b runs unit b, its warp w runs round w of it --
-// the same arithmetic as the persistent kernel, spread over more warps.
+// Plain per-phase kernels, with the same arithmetic as the persistent kernel.
+// Setup: each warp runs one unit (8 per block).  Shading: block b runs unit
+// b, its warp w runs round w of it.
 __global__ void __launch_bounds__(kThreads) k_setup(TableRef tb, int item) {
   const DItem& it = tb.items[item];
   const int u = blockIdx.x * kWarps + (threadIdx.x >> 5);
   if (u < it.units[PH_SETUP]) unit_setup(it, tb.shells + it.shell0, u);
 }
 
+// Raster: resident blocks only, every warp strides over the item's units (of
+// 32 triangles, or fewer where the mesh is too small to give every warp
+// one: see raster_shape).  What bounds it: latency of the dependent index and
+// vertex loads and of the walk.  One block per 256 triangles, each of its
+// warps adding its counts to the workspace header by itself, made 87 k
+// atomics on one cache line of an 800^2 view of 7 x 200 k triangles, and they
+// were the kernel's time; now a block adds its counts once.
 template <bool FULL>
-__global__ void __launch_bounds__(kThreads) k_raster(TableRef tb, int item) {
+__global__ void __launch_bounds__(kThreads, kRasterBlocks) k_raster(TableRef tb, int item) {
+  __shared__ unsigned s_count[7];
   const DItem& it = tb.items[item];
+  const DShell* sh = tb.shells + it.shell0;
   const int w = threadIdx.x >> 5;
-  unit_raster<FULL>(it, tb.shells + it.shell0, blockIdx.x, tb.hdr, vs_smem + w * kRasterWarpBytes, w, w + 1);
+  if (threadIdx.x < 7) s_count[threadIdx.x] = 0;
+  __syncthreads();
+  RasterCounts rc = {0, 0, 0, 0};
+  for (int u = blockIdx.x * kWarps + w; u < it.units[PH_RASTER]; u += gridDim.x * kWarps)
+    unit_raster<FULL>(it, sh, u, vs_smem + w * kRasterWarpBytes, rc);
+  const unsigned c[7] = {rc.fb & 0xFFFFu, rc.fb >> 16, rc.ng & 0xFFFFu, rc.ng >> 16, rc.lc & 0xFFFFu, rc.lc >> 16,
+                         rc.bad};
+#pragma unroll
+  for (int q = 0; q < 7; ++q) {
+    const unsigned v = __reduce_add_sync(0xffffffffu, c[q]);
+    if ((threadIdx.x & 31) == 0 && v) atomicAdd(&s_count[q], v);
+  }
+  __syncthreads();
+  if (threadIdx.x < 6 && s_count[threadIdx.x]) {
+    WsHeader* h = tb.hdr;
+    unsigned long long* dst[6] = {&h->front, &h->back, &h->nearc, &h->guard, &h->large, &h->clipped};
+    atomicAdd(dst[threadIdx.x], (unsigned long long)s_count[threadIdx.x]);
+  }
+  if (threadIdx.x == 6 && s_count[6]) record_error(tb.hdr, VS_ERR_INVALID_ARG);
 }
 
 }  // namespace vsd
@@ -64,12 +91,13 @@ cudaError_t upload(char* ws, const UploadChunk& c, cudaStream_t st) {
 int plain_forward_launches(const int units[4]) { return (units[0] > 0) + (units[1] > 0) + (units[2] > 0); }
 int plain_backward_launches(const int units[4]) { return (units[0] > 0) + (units[2] > 0); }
 
-cudaError_t plain_forward(const TableRef& tb, const int units[4], int tc, bool full, cudaStream_t st) {
+cudaError_t plain_forward(const TableRef& tb, const int units[4], int tc, bool full, int sms, cudaStream_t st) {
   const int W = vsd::kWarps;
   if (units[0]) vsd::k_setup<<<(units[0] + W - 1) / W, vsd::kThreads, 0, st>>>(tb, 0);
   if (units[1]) {
-    if (full) vsd::k_raster<true><<<units[1], vsd::kThreads, vsd::kRasterWarpBytes * W, st>>>(tb, 0);
-    else vsd::k_raster<false><<<units[1], vsd::kThreads, vsd::kRasterWarpBytes * W, st>>>(tb, 0);
+    const int grid = std::min((units[1] + W - 1) / W, sms * vsd::kRasterBlocks);
+    if (full) vsd::k_raster<true><<<grid, vsd::kThreads, vsd::kRasterWarpBytes * W, st>>>(tb, 0);
+    else vsd::k_raster<false><<<grid, vsd::kThreads, vsd::kRasterWarpBytes * W, st>>>(tb, 0);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || !units[2]) return e;

@@ -70,17 +70,19 @@ static __device__ void unit_setup(const DItem& it, const DShell* sh, int u) {
 // ----------------------------------------------------------------------------
 // RASTER
 // ----------------------------------------------------------------------------
-// Loads triangle t of shell s; 0 = front-facing and rasterizable, 1..3 =
-// culled (back/zero-area, behind the near plane, guard band), 4 = index out
-// of range, 5 = to be clipped at the near plane.
-__device__ __forceinline__ int load_tri(const DShell& s, const DCam& c, int t, Tri& T, int idx[3]) {
-  const int* ip = s.tris + 3 * (size_t)t;
-  idx[0] = __ldg(ip);
-  idx[1] = __ldg(ip + 1);
-  idx[2] = __ldg(ip + 2);
-  if ((unsigned)idx[0] >= (unsigned)s.nv || (unsigned)idx[1] >= (unsigned)s.nv || (unsigned)idx[2] >= (unsigned)s.nv)
+// Vertex indices of triangle t (garbage-free for t >= nt: triangle nt - 1).
+__device__ __forceinline__ int3 load_index(const DShell& s, int t) {
+  const int* ip = s.tris + 3 * (size_t)min(t, s.nt - 1);
+  return make_int3(__ldg(ip), __ldg(ip + 1), __ldg(ip + 2));
+}
+
+// The triangle of vertices ix in shell s; 0 = front-facing and rasterizable,
+// 1..3 = culled (back/zero-area, behind the near plane, guard band), 4 =
+// index out of range, 5 = to be clipped at the near plane.
+__device__ __forceinline__ int load_tri(const DShell& s, const DCam& c, const int3 ix, Tri& T) {
+  if ((unsigned)ix.x >= (unsigned)s.nv || (unsigned)ix.y >= (unsigned)s.nv || (unsigned)ix.z >= (unsigned)s.nv)
     return 4;
-  return make_tri(__ldcg(s.vsetup + idx[0]), __ldcg(s.vsetup + idx[1]), __ldcg(s.vsetup + idx[2]), c.W, c.H, T);
+  return make_tri(__ldcg(s.vsetup + ix.x), __ldcg(s.vsetup + ix.y), __ldcg(s.vsetup + ix.z), c.W, c.H, T);
 }
 
 __device__ __forceinline__ void raster_pixel(const Tri& T, int t, int x, int y, int W, unsigned long long* vis) {
@@ -90,18 +92,19 @@ __device__ __forceinline__ void raster_pixel(const Tri& T, int t, int x, int y, 
 }
 
 // The parts of triangle t clipped at the near plane, rasterized by the whole
-// warp (each lane strides over the parts' screen boxes).  Rare: out of line.
-static __device__ __forceinline__ void raster_clipped(const DShell& s, const DCam& c, int t, unsigned long long* vis) {
+// warp (each lane strides over the parts' screen boxes; warps that share a
+// round take every `step`-th pixel from `first` on).  Rare: out of line.
+static __device__ __forceinline__ void raster_clipped(const DShell& s, const DCam& c, int t, unsigned long long* vis,
+                                                      int first, int step) {
   const int* ip = s.tris + 3 * (size_t)t;
   const int idx[3] = {__ldg(ip), __ldg(ip + 1), __ldg(ip + 2)};   // checked in range by load_tri
   Tri part[2];
   float2 puv[2][3];
   const int np = clip_tri(s.pos, nullptr, c, idx, part, puv);
-  const int lane = threadIdx.x & 31;
   for (int k = 0; k < np; ++k) {
     const int bw = part[k].xhi - part[k].xlo + 1, bh = part[k].yhi - part[k].ylo + 1;
     const int npq = bw > 0 && bh > 0 ? bw * bh : 0;
-    for (int p = lane; p < npq; p += 32) {
+    for (int p = first; p < npq; p += step) {
       const int yy = p / bw;
       raster_pixel(part[k], t, part[k].xlo + (p - yy * bw), part[k].ylo + yy, c.W, vis);
     }
@@ -109,9 +112,13 @@ static __device__ __forceinline__ void raster_clipped(const DShell& s, const DCa
 }
 
 // Triangle record shared by the lanes of a warp during the raster walk.
-// Small boxes (<= kSmallMaxPixels pixel centres) keep every edge function
-// value within +-2^30, so the walk runs in 32-bit integers: e_j(dx, dy) =
-// c_j + gx_j dx + gy_j dy for pixel (xlo + dx, ylo + dy).
+// Triangles less than 64 pixels wide and high (kNarrow, before clipping the
+// box to the image) keep every edge function value within +-2^29, so the
+// walk runs in 32-bit integers: e_j(dx, dy) = c_j + gx_j dx + gy_j dy for
+// pixel (xlo + dx, ylo + dy).  The bound is on the triangle's extent and not
+// on the pixels of its box: a 14 x 14 pixel triangle of a coarse mesh walks
+// with the others of its round (it used to be walked alone, in 64 bits).
+constexpr int kNarrow = 64 * 256;
 struct TriS {
   int c[3], gx[3], gy[3];
   unsigned q[3];
@@ -124,8 +131,11 @@ struct TriPos {        // box origin of a record
   int xlo, ylo;
 };
 
-// floor(sum_j e_j q_j / S) for the 32-bit edge values of a small box; same
-// estimate-and-correct scheme as depth_key_r.
+// floor(sum_j e_j q_j / S) for the 32-bit edge values of a narrow triangle;
+// same estimate-and-correct scheme as depth_key_r.  The estimate is within
+// ~640 of the quotient, so |R| < 2^10 S: from S = 2^21 on R is taken to FP32
+// in units of 2^10 (a thousandth of S), below it fits 32 bits.  (A 64-bit
+// integer converted to FP32 runs on the FP64 pipe, a 64th of the FP32 rate.)
 __device__ __forceinline__ unsigned depth_key32(const unsigned q[3], const int e[3], int S, float rS) {
   const unsigned long long N = (unsigned long long)(unsigned)e[0] * q[0] +
                                (unsigned long long)(unsigned)e[1] * q[1] +
@@ -135,8 +145,10 @@ __device__ __forceinline__ unsigned depth_key32(const unsigned q[3], const int e
   unsigned Q = (unsigned)fminf(fmaxf(est, (float)qmin), (float)qmax);
   Q = min(max(Q, qmin), qmax);
   long long R = (long long)(N - (unsigned long long)Q * (unsigned)S);
-  Q = (unsigned)((long long)Q + (long long)floorf((float)R * rS));
-  R = (long long)(N - (unsigned long long)Q * (unsigned)S);
+  const bool big = S >= (1 << 21);
+  const int dQ = (int)floorf((float)(int)(R >> (big ? 10 : 0)) * (big ? 1024.0f * rS : rS));
+  Q += (unsigned)dQ;
+  R -= (long long)dQ * S;
 #pragma unroll 1
   for (int i = 0; i < 4 && R < 0; ++i) { --Q; R += S; }
 #pragma unroll 1
@@ -144,43 +156,51 @@ __device__ __forceinline__ unsigned depth_key32(const unsigned q[3], const int e
   return Q;
 }
 
-// Per-lane triangle counts of a raster unit, two 16-bit fields per word (a
-// lane sees one triangle per round and a unit has at most 2048 / 32 = 64
-// rounds, so no field overflows): fb = front | back << 16, ng = near plane |
-// guard band << 16, lc = large box | clipped << 16, plus an error bit.
+// Per-lane triangle counts of a raster unit (or of a warp of the plain
+// kernel), two 16-bit fields per word (a lane sees one triangle per round; a
+// unit has at most 2048 / 32 = 64 rounds and a warp of the plain kernel at
+// most 16 2^27 / 32 / (24 per SM) = 2^18 / 7 on a GPU of 76 SMs or more, so no
+// field overflows): fb = front | back << 16, ng = near plane | guard band <<
+// 16, lc = box over 64 pixels | clipped << 16, plus an error bit.
 struct RasterCounts {
   unsigned fb, ng, lc, bad;
 };
+constexpr int kLargePixels = 64;   // vs_stats.tris_large
 
-// One round of a raster unit: 32 triangles t0 + lane of one shell.  Each
-// lane sets up one triangle; then the warp walks all (triangle, box pixel)
-// pairs of the 32 triangles together: window by window, a warp-wide OR of
-// the triangles' start bits tells every lane which triangle owns its pair,
-// so lanes do not idle on small or culled boxes.  Larger boxes are
-// rasterized by the whole warp, one triangle at a time.
+// One round of a raster unit: up to 32 triangles t0 + lane < tend of one
+// shell, whose indices ix the caller has loaded.  Each lane sets up one
+// triangle; then the warp walks all (triangle, box pixel) pairs of the
+// round's narrow triangles together: window by window, a warp-wide OR of the
+// triangles' start bits tells every lane which triangle owns its pair, so
+// lanes do not idle on small or culled boxes.  Wider triangles are
+// rasterized by the whole warp, one at a time, in 64 bits.  A round of one
+// triangle may be shared by 2^lg warps: warp `part` takes every 2^lg-th
+// window.
 template <bool FULL>
-__device__ __forceinline__ void raster_round(const DItem& it, const DShell& s, int t0, unsigned long long* vis,
-                                             char* smem, RasterCounts& rc) {
+__device__ __forceinline__ void raster_round(const DItem& it, const DShell& s, int t0, int tend, const int3 ix, int part,
+                                             int lg, unsigned long long* vis, char* smem, RasterCounts& rc) {
   TriS* s_tri = reinterpret_cast<TriS*>(smem);
   TriPos* s_pos = reinterpret_cast<TriPos*>(smem + sizeof(TriS) * 32);
   int* s_start = reinterpret_cast<int*>(smem + (sizeof(TriS) + sizeof(TriPos)) * 32);
   const unsigned kAll = 0xffffffffu;
-  const int lane = threadIdx.x & 31, wbase = 0;
+  const int lane = threadIdx.x & 31;
   const int t = t0 + lane;
   const int W = it.cam.W;
-  unsigned front = 0, back = 0, nearc = 0, guard = 0, large = 0, bad = 0, clip = 0;
+  unsigned front = 0, back = 0, nearc = 0, guard = 0, large = 0, bad = 0, clip = 0, wide = 0;
   int npx = 0;
   TriS r;
   TriPos pos;
-  if (t < s.nt) {
+  if (t < tend) {
     Tri T;
-    int idx[3];
-    const int why = load_tri(s, it.cam, t, T, idx);
+    const int why = load_tri(s, it.cam, ix, T);
     if (why == 0) {
       front = 1;
       const int bw = T.xhi - T.xlo + 1, bh = T.yhi - T.ylo + 1;
       if (bw > 0 && bh > 0) {
-        if (bw * bh <= kSmallMaxPixels) {
+        large = bw * bh > kLargePixels;
+        const int ext = max(max(max(T.X[0], T.X[1]), T.X[2]) - min(min(T.X[0], T.X[1]), T.X[2]),
+                            max(max(T.Y[0], T.Y[1]), T.Y[2]) - min(min(T.Y[0], T.Y[1]), T.Y[2]));
+        if (ext < kNarrow) {
           npx = bw * bh;
           const int ox = 256 * T.xlo + 128, oy = 256 * T.ylo + 128;
           int S = 0;
@@ -203,7 +223,7 @@ __device__ __forceinline__ void raster_round(const DItem& it, const DShell& s, i
           pos.xlo = T.xlo;
           pos.ylo = T.ylo;
         } else {
-          large = 1;
+          wide = 1;
         }
       }
     } else if (why == 1) back = 1;
@@ -214,63 +234,66 @@ __device__ __forceinline__ void raster_round(const DItem& it, const DShell& s, i
   }
   // compact the non-empty boxes and take the exclusive prefix of their sizes
   const unsigned ne = __ballot_sync(kAll, npx > 0);
-  int pre = npx;
+  if (ne) {
+    int pre = npx;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(kAll, pre, o);
-    if (lane >= o) pre += v;
-  }
-  const int total = __shfl_sync(kAll, pre, 31);
-  const int start = pre - npx;
-  if (npx > 0) {
-    const int cpos = __popc(ne & ((1u << lane) - 1u));
-    s_tri[wbase + cpos] = r;
-    s_pos[wbase + cpos] = pos;
-    s_start[wbase + cpos] = start;
-  }
-  __syncwarp();
-  const unsigned le = (lane == 31) ? kAll : ((2u << lane) - 1u);
-  int carry = 0;
-  for (int w0 = 0; w0 < total; w0 += 32) {
-    const unsigned b = (npx > 0 && start >= w0 && start < w0 + 32) ? (1u << (start - w0)) : 0u;
-    const unsigned bits = __reduce_or_sync(kAll, b);
-    const int slot = w0 + lane;
-    if (slot < total) {
-      const int o = carry + __popc(bits & le) - 1;
-      const TriS& q = s_tri[wbase + o];
-      const int local = slot - s_start[wbase + o];
-      const int bwq = q.tl_bw >> 8;
-      const int dy = (int)(((float)local + 0.5f) * q.rbw);
-      const int dx = local - dy * bwq;
-      int e[3];
-#pragma unroll
-      for (int j = 0; j < 3; ++j) e[j] = q.c[j] + q.gx[j] * dx + q.gy[j] * dy;
-      if ((e[0] + (q.tl_bw & 1) > 0) && (e[1] + ((q.tl_bw >> 1) & 1) > 0) && (e[2] + ((q.tl_bw >> 2) & 1) > 0)) {
-        const TriPos p = s_pos[wbase + o];
-        const int S = e[0] + e[1] + e[2];
-        red_max_vis(vis + (size_t)(p.ylo + dy) * W + (p.xlo + dx), vis_key(depth_key32(q.q, e, S, q.rS), q.t));
-      }
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(kAll, pre, o);
+      if (lane >= o) pre += v;
     }
-    carry += __popc(bits);
+    const int total = __shfl_sync(kAll, pre, 31);
+    const int start = pre - npx;
+    if (npx > 0) {
+      const int cpos = __popc(ne & ((1u << lane) - 1u));
+      s_tri[cpos] = r;
+      s_pos[cpos] = pos;
+      s_start[cpos] = start;
+    }
+    __syncwarp();
+    const unsigned le = (lane == 31) ? kAll : ((2u << lane) - 1u);
+    int carry = 0;
+    for (int w0 = 32 * part; w0 < total; w0 += 32 << lg) {
+      const unsigned b = (npx > 0 && start >= w0 && start < w0 + 32) ? (1u << (start - w0)) : 0u;
+      const unsigned bits = __reduce_or_sync(kAll, b);
+      const int slot = w0 + lane;
+      if (slot < total) {
+        const int o = lg ? 0 : carry + __popc(bits & le) - 1;
+        const TriS& q = s_tri[o];
+        const int local = slot - s_start[o];
+        const int bwq = q.tl_bw >> 8;
+        const int dy = (int)(((float)local + 0.5f) * q.rbw);
+        const int dx = local - dy * bwq;
+        int e[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) e[j] = q.c[j] + q.gx[j] * dx + q.gy[j] * dy;
+        if ((e[0] + (q.tl_bw & 1) > 0) && (e[1] + ((q.tl_bw >> 1) & 1) > 0) && (e[2] + ((q.tl_bw >> 2) & 1) > 0)) {
+          const TriPos p = s_pos[o];
+          const int S = e[0] + e[1] + e[2];
+          red_max_vis(vis + (size_t)(p.ylo + dy) * W + (p.xlo + dx), vis_key(depth_key32(q.q, e, S, q.rS), q.t));
+        }
+      }
+      carry += __popc(bits);
+    }
   }
-  rc.fb += front | (back << 16);
-  rc.ng += nearc | (guard << 16);
-  rc.lc += large | (clip << 16);
+  if (part == 0) {
+    rc.fb += front | (back << 16);
+    rc.ng += nearc | (guard << 16);
+    rc.lc += large | (clip << 16);
+  }
   rc.bad |= bad;
-  // large boxes: the warp strides over each one's screen box
-  unsigned lm = __ballot_sync(kAll, large);
+  // wide triangles: the warp strides over each one's screen box
+  unsigned lm = __ballot_sync(kAll, wide);
   while (lm) {
     const int l = __ffs(lm) - 1;
     lm &= lm - 1;
-    const int tq = __shfl_sync(kAll, t, l);
+    const int3 iq = make_int3(__shfl_sync(kAll, ix.x, l), __shfl_sync(kAll, ix.y, l), __shfl_sync(kAll, ix.z, l));
     Tri T;
-    int idx[3];
-    if (load_tri(s, it.cam, tq, T, idx) != 0) continue;
+    if (load_tri(s, it.cam, iq, T) != 0) continue;
     const int bw = T.xhi - T.xlo + 1, bh = T.yhi - T.ylo + 1;
     const int npq = bw * bh;
-    for (int p = lane; p < npq; p += 32) {
+    for (int p = 32 * part + lane; p < npq; p += 32 << lg) {
       const int yy = p / bw;
-      raster_pixel(T, tq, T.xlo + (p - yy * bw), T.ylo + yy, W, vis);
+      raster_pixel(T, t0 + l, T.xlo + (p - yy * bw), T.ylo + yy, W, vis);
     }
   }
   // triangles clipped at the near plane (items with a vertex nearer than
@@ -280,33 +303,33 @@ __device__ __forceinline__ void raster_round(const DItem& it, const DShell& s, i
     while (cm) {
       const int l = __ffs(cm) - 1;
       cm &= cm - 1;
-      raster_clipped(s, it.cam, __shfl_sync(kAll, t, l), vis);
+      raster_clipped(s, it.cam, __shfl_sync(kAll, t, l), vis, 32 * part + lane, 32 << lg);
     }
   }
   __syncwarp();   // the records are reused by the next round
 }
 
-// Raster unit: 32 * it.raster_rounds triangles of one shell in rounds of 32;
-// this warp runs rounds [r0, r1).
+// Raster unit u: it.raster_tris consecutive triangles of one shell in rounds
+// of 32 (or one triangle shared by 2^raster_lg units).  The next round's
+// indices are loaded while the current one runs.
 template <bool FULL>
-static __device__ __forceinline__ void unit_raster(const DItem& it, const DShell* sh, int u, WsHeader* hdr, char* smem,
-                                                   int r0, int r1) {
+static __device__ __forceinline__ void unit_raster(const DItem& it, const DShell* sh, int u, char* smem,
+                                                   RasterCounts& rc) {
+  const int lg = it.raster_lg, part = u & ((1 << lg) - 1);
+  u >>= lg;
   int i = 0;
   while (i + 1 < it.k && u >= it.raster_pre[i + 1]) ++i;
   const DShell& s = sh[i];
-  const int per_unit = 32 * it.raster_rounds;
-  const int base = (u - it.raster_pre[i]) * per_unit;
+  const int base = (u - it.raster_pre[i]) * it.raster_tris;
+  const int end = min(s.nt, base + it.raster_tris);
   unsigned long long* vis = it.vis + (size_t)i * it.cam.W * it.cam.H;
-  RasterCounts rc = {0, 0, 0, 0};
-  const int rounds = min(r1, min(per_unit, s.nt - base + 31) / 32);
-  for (int r = r0; r < rounds; ++r) raster_round<FULL>(it, s, base + 32 * r, vis, smem, rc);
-  warp_count(&hdr->front, rc.fb & 0xFFFFu);
-  warp_count(&hdr->back, rc.fb >> 16);
-  warp_count(&hdr->nearc, rc.ng & 0xFFFFu);
-  warp_count(&hdr->guard, rc.ng >> 16);
-  warp_count(&hdr->large, rc.lc & 0xFFFFu);
-  warp_count(&hdr->clipped, rc.lc >> 16);
-  if (__any_sync(0xffffffffu, rc.bad) && (threadIdx.x & 31) == 0) record_error(hdr, VS_ERR_INVALID_ARG);
+  const int lane = threadIdx.x & 31;
+  int3 ix = load_index(s, base + lane);
+  for (int t0 = base; t0 < end; t0 += 32) {
+    const int3 cur = ix;
+    if (t0 + 32 < end) ix = load_index(s, t0 + 32 + lane);
+    raster_round<FULL>(it, s, t0, end, cur, part, lg, vis, smem, rc);
+  }
 }
 
 // ----------------------------------------------------------------------------
@@ -1068,7 +1091,18 @@ __global__ void __launch_bounds__(pers_threads(BWD), BWD ? VS_PERS_BWD_BLOCKS : 
     const DShell* sh = tb.shells + it.shell0;
     switch (ph) {
       case PH_SETUP: unit_setup(it, sh, u); break;
-      case PH_RASTER: unit_raster<FULL>(it, sh, u, hdr, smem, 0, it.raster_rounds); break;
+      case PH_RASTER: {
+        RasterCounts rc = {0, 0, 0, 0};
+        unit_raster<FULL>(it, sh, u, smem, rc);
+        warp_count(&hdr->front, rc.fb & 0xFFFFu);
+        warp_count(&hdr->back, rc.fb >> 16);
+        warp_count(&hdr->nearc, rc.ng & 0xFFFFu);
+        warp_count(&hdr->guard, rc.ng >> 16);
+        warp_count(&hdr->large, rc.lc & 0xFFFFu);
+        warp_count(&hdr->clipped, rc.lc >> 16);
+        if (__any_sync(kAll, rc.bad) && lane == 0) record_error(hdr, VS_ERR_INVALID_ARG);
+        break;
+      }
       default:
         unit_shade<BWD, false, TC, FULL>(it, sh, u, hdr, smem, tb.kmax, 0, it.shade_rounds);
     }

@@ -54,7 +54,7 @@ extern const TcOps kTcAny, kTcRgba, kTcSh0, kTcSh1, kTcSh2, kTcSh3, kTcU80, kTcU
 cudaError_t upload(char* ws, const UploadChunk& c, cudaStream_t st);
 int plain_forward_launches(const int units[4]);
 int plain_backward_launches(const int units[4]);
-cudaError_t plain_forward(const TableRef& tb, const int units[4], int tc, bool full, cudaStream_t st);
+cudaError_t plain_forward(const TableRef& tb, const int units[4], int tc, bool full, int sms, cudaStream_t st);
 cudaError_t plain_backward(const TableRef& tb, const int units[4], int tc, bool full, cudaStream_t st);
 cudaError_t persistent(const TableRef& tb, bool bwd, int tc, bool full, int grid, long long spin_limit,
                        cudaStream_t st);

@@ -234,11 +234,13 @@ void order_for_locality(std::vector<ItemReq>& req) {
 
 // Work-unit sizes of one plan: the most triangles per raster unit, the 32-wide
 // rounds per shading unit (the plain launch runs one per warp of a block),
-// and the warps that should find a raster unit (those resident on the GPU).
+// and the warps that should find a raster unit (those resident on the GPU)
+// and a setup unit.
 struct UnitShape {
   int raster_tris = 32;
   int shade_rounds = kWarps;
   int warps = 0;
+  int setup_warps = 0;
 };
 
 // Raster units of an item of `tris` triangles: units of the asked size while
@@ -251,6 +253,20 @@ void raster_shape(long long tris, const UnitShape& shape, int* unit, int* lg) {
   *lg = 0;
   while (*unit > 1 && tris / *unit < shape.warps) *unit /= 2;
   while (*unit == 1 && *lg < 6 && (tris << (*lg + 1)) <= shape.warps) ++*lg;
+}
+
+// Setup units of an item of `verts` vertices and `words` visibility words to
+// clear: the largest size at which every warp asked for finds one of each
+// kind, but no fewer than 32 vertices (one per lane) and 512 words (8 stores
+// of 512 bytes).  At the largest size, 1024 vertices one after the other per
+// lane were the critical path of a single view: 25 us for the setup of an
+// 800^2 view of 7 x 200 k triangles, and as much for
+// that of a 256^2 view of 3 x 1.2 k, which takes 2.5 us in small units.
+void setup_shape(long long verts, long long words, const UnitShape& shape, int* uv, int* uw) {
+  *uv = kSetupVerts;
+  *uw = kClearWords;
+  while (*uv > 32 && verts / *uv < shape.setup_warps) *uv /= 2;
+  while (*uw > 512 && words / *uw < shape.setup_warps) *uw /= 2;
 }
 
 struct Plan {
@@ -355,12 +371,16 @@ vs_status make_plan(const ItemReq* req, int n, const float* bg, int do_bwd, bool
     it.flags = (int)flags;
     it.do_bwd = do_bwd;
     it.stall = (flags & VS_FLAG_TEST_STALL) ? 1 : 0;
-    long long tris = 0;
-    for (int i = 0; i < o.k; ++i) tris += o.shells[i].num_tris;
+    long long tris = 0, verts = 0;
+    for (int i = 0; i < o.k; ++i) {
+      tris += o.shells[i].num_tris;
+      verts += o.shells[i].num_verts;
+    }
     raster_shape(tris, shape, &it.raster_tris, &it.raster_lg);
     it.shade_rounds = shape.shade_rounds;
     it.bg[0] = bg ? bg[0] : 0.f; it.bg[1] = bg ? bg[1] : 0.f; it.bg[2] = bg ? bg[2] : 0.f;
     const size_t HW = (size_t)c.width * c.height;
+    setup_shape(verts, (long long)(o.k * HW), shape, &it.setup_verts, &it.clear_words);
     it.setup_pre[0] = 0;
     it.raster_pre[0] = 0;
     for (int i = 0; i < o.k; ++i) {
@@ -393,13 +413,13 @@ vs_status make_plan(const ItemReq* req, int n, const float* bg, int do_bwd, bool
       }
       s.vsetup = reinterpret_cast<int4*>(ws ? ws + off : nullptr);
       off = align256(off + sizeof(int4) * (size_t)d.num_verts);
-      it.setup_pre[i + 1] = it.setup_pre[i] + (d.num_verts + kSetupPerUnit - 1) / kSetupPerUnit;
+      it.setup_pre[i + 1] = it.setup_pre[i] + (d.num_verts + it.setup_verts - 1) / it.setup_verts;
       it.raster_pre[i + 1] = it.raster_pre[i] + (d.num_tris + it.raster_tris - 1) / it.raster_tris;
     }
     it.vis = reinterpret_cast<unsigned long long*>(ws ? ws + off : nullptr);
     if (clear_vis) off = align256(off + sizeof(unsigned long long) * o.k * HW);
     const size_t vis_words = (size_t)o.k * HW;
-    it.clear_units = clear_vis ? (int)((vis_words + kClearPerUnit - 1) / kClearPerUnit) : 0;
+    it.clear_units = clear_vis ? (int)((vis_words + it.clear_words - 1) / it.clear_words) : 0;
     it.units[PH_SETUP] = it.clear_units + it.setup_pre[o.k];
     it.units[PH_RASTER] = clear_vis ? it.raster_pre[o.k] << it.raster_lg : 0;
     it.units[PH_SHADE] = (int)((HW + shade_per_unit - 1) / shade_per_unit);
@@ -535,7 +555,7 @@ int resident_warps(const vs_ctx* ctx) { return ctx->num_sms * kRasterBlocks * kW
 
 UnitShape plain_shape(const vs_ctx* ctx) {
   UnitShape u;
-  u.warps = resident_warps(ctx);
+  u.warps = u.setup_warps = resident_warps(ctx);
   return u;
 }
 
@@ -824,7 +844,7 @@ vs_status vs_render_backward(vs_ctx* ctx, const vs_object* obj, const vs_camera*
   char* ws = static_cast<char*>(workspace);
   if ((s = set_device(ctx)) != VS_OK) return s;
   if ((s = ensure_bounds(obj)) != VS_OK) return s;
-  if ((s = make_plan(&r, 1, bg, 1, false, flags & ~VS_FLAG_TEST_STALL, ws, P)) != VS_OK) return s;
+  if ((s = make_plan(&r, 1, bg, 1, false, flags & ~VS_FLAG_TEST_STALL, ws, P, plain_shape(ctx))) != VS_OK) return s;
   if ((s = check_ws(P, workspace, ws_bytes)) != VS_OK) return s;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if ((s = upload_table(P, ws, vsk::plain_backward_launches(P.items[0].units), st)) != VS_OK) return s;

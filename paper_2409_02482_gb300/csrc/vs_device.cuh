@@ -20,8 +20,8 @@ namespace vsd {
 // ----------------------------------------------------------------------------
 constexpr int kThreads = 256;          // threads per block, all kernels
 constexpr int kWarps = kThreads / 32;  // a work unit is run by one warp
-constexpr int kSetupPerUnit = 1024;    // vertices per setup unit
-constexpr int kClearPerUnit = 16384;   // visibility words cleared per unit
+constexpr int kSetupVerts = 1024;      // most vertices per setup unit
+constexpr int kClearWords = 16384;     // most visibility words cleared per unit
 constexpr int kShadePixels = 256;      // pixels per shading unit of the plain launches
 // The plain shading launch runs one unit per block, one 32-wide round per
 // warp, so its units are kWarps rounds; the persistent kernel takes any size
@@ -150,6 +150,8 @@ struct alignas(16) DItem {
   int32_t flags, do_bwd, stall;
   int32_t raster_tris;         // triangles per raster unit (a power of two)
   int32_t shade_rounds;        // shading unit = 32 * shade_rounds pixels
+  int32_t setup_verts;         // vertices per setup unit
+  int32_t clear_words;         // visibility words per clearing unit (even)
   int32_t units[4];            // per phase (3 used)
   int32_t setup_pre[kMaxShells + 1];
   int32_t raster_pre[kMaxShells + 1];

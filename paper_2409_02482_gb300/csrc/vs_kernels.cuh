@@ -50,8 +50,8 @@ namespace vsd {
 static __device__ void unit_setup(const DItem& it, const DShell* sh, int u) {
   if (u < it.clear_units) {
     const size_t total = (size_t)it.k * it.cam.W * it.cam.H;
-    const size_t beg = (size_t)u * kClearPerUnit;
-    const size_t end = min(total, beg + (size_t)kClearPerUnit);
+    const size_t beg = (size_t)u * it.clear_words;
+    const size_t end = min(total, beg + (size_t)it.clear_words);
     uint4* p = reinterpret_cast<uint4*>(it.vis + beg);
     const size_t n2 = (end - beg) >> 1;
     for (size_t i = threadIdx.x & 31; i < n2; i += 32) clear_vis2(p + i);
@@ -62,8 +62,8 @@ static __device__ void unit_setup(const DItem& it, const DShell* sh, int u) {
   int i = 0;
   while (i + 1 < it.k && u >= it.setup_pre[i + 1]) ++i;
   const DShell& s = sh[i];
-  const int v0 = (u - it.setup_pre[i]) * kSetupPerUnit;
-  const int v1 = min(v0 + kSetupPerUnit, s.nv);
+  const int v0 = (u - it.setup_pre[i]) * it.setup_verts;
+  const int v1 = min(v0 + it.setup_verts, s.nv);
   for (int v = v0 + (threadIdx.x & 31); v < v1; v += 32) s.vsetup[v] = setup_vertex(s.pos + 3 * (size_t)v, it.cam);
 }
 

@@ -9,6 +9,7 @@
 #pragma once
 
 #include <cuda_fp16.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include "vs.h"
@@ -160,20 +161,22 @@ struct alignas(16) DItem {
 
 // Workspace header (first 256 bytes).  status and the counters persist
 // across calls until vs_read_stats resets them; next_unit and abort are
-// reset by every call's table upload.
+// reset by every call's table upload.  next_unit has a 128-byte line of its
+// own: atomics on one line go one after the other (about 2.5 ns each), and
+// the persistent kernel's warps take every unit there.
 struct alignas(16) WsHeader {
   int32_t status;
   int32_t abort;
-  uint32_t next_unit;
-  int32_t pad;
+  int32_t pad[2];
   unsigned long long frags, front, back, nearc, guard, large;
   unsigned long long launches;  // kernels enqueued by the calls (host-declared)
   unsigned long long clipped;   // triangles clipped at the near plane
   int32_t kernel_class;         // shading kernels of the last call (host-declared)
-  int32_t pad1;
-  unsigned long long reserved[21];
+  int32_t pad1[11];
+  uint32_t next_unit;
+  int32_t reserved[31];
 };
-static_assert(sizeof(WsHeader) == 256, "header is 256 bytes");
+static_assert(sizeof(WsHeader) == 256 && offsetof(WsHeader, next_unit) == 128, "header layout");
 
 // ----------------------------------------------------------------------------
 // small helpers

@@ -988,9 +988,10 @@ __device__ __forceinline__ void shade_round(const DItem& it, const DShell* sh, i
 
 // Shading unit: 32 * it.shade_rounds consecutive pixels in rounds of 32;
 // this warp runs rounds [r0, r1).  `wb` is the warp's shared-memory slice.
+// Returns the lane's shaded fragments.
 template <bool BWD, bool FROM_HITS, int TC, bool FULL>
-__device__ __forceinline__ void unit_shade(const DItem& it, const DShell* sh, int u, WsHeader* hdr, char* wb, int K,
-                                           int r0, int r1) {
+__device__ __forceinline__ unsigned unit_shade(const DItem& it, const DShell* sh, int u, WsHeader* hdr, char* wb, int K,
+                                               int r0, int r1) {
   const unsigned kAll = 0xffffffffu;
   const int HW = it.cam.W * it.cam.H;
   unsigned nfrag = 0, bad = 0;
@@ -1001,7 +1002,6 @@ __device__ __forceinline__ void unit_shade(const DItem& it, const DShell* sh, in
     shade_round<BWD, FROM_HITS, TC, FULL>(it, sh, pbase, wb, K, nfrag, bad, loss);
   }
   const int lane = threadIdx.x & 31;
-  if (!FROM_HITS) warp_count(&hdr->frags, nfrag);
   if (__any_sync(kAll, bad) && lane == 0) record_error(hdr, VS_ERR_INVALID_ARG);
   if constexpr (BWD) {
     if (it.loss && (it.flags & (VS_FLAG_LOSS_L2 | VS_FLAG_LOSS_L1))) {
@@ -1010,6 +1010,7 @@ __device__ __forceinline__ void unit_shade(const DItem& it, const DShell* sh, in
       if (lane == 0 && loss != 0.0f) atomicAdd(it.loss, loss);
     }
   }
+  return nfrag;
 }
 
 extern __shared__ __align__(16) char vs_smem[];
@@ -1021,22 +1022,50 @@ __device__ __forceinline__ char* warp_smem(int K, bool bwd, int tc) {
 
 template <bool BWD, bool FROM_HITS, int TC, bool FULL>
 __global__ void __launch_bounds__(kThreads, BWD ? VS_BWD_BLOCKS : VS_FWD_BLOCKS) k_shade(TableRef tb, int item) {
+  __shared__ unsigned s_frags;
   const DItem& it = tb.items[item];
   const int w = threadIdx.x >> 5;
-  unit_shade<BWD, FROM_HITS, TC, FULL>(it, tb.shells + it.shell0, blockIdx.x, tb.hdr, warp_smem(tb.kmax, BWD, TC), tb.kmax, w,
-                             w + 1);
+  // One addition per warp is 20 k atomics on one word for an 800^2 view (SH2:
+  // 194.5 us a frame, 190.9 with one per block).  The baked classes keep it:
+  // their 1080p frame takes 389.9 us, and 395 with the block's sum.
+  constexpr bool kBlockCount = !FROM_HITS && TC < TC_U80;
+  if (kBlockCount) {
+    if (threadIdx.x == 0) s_frags = 0;
+    __syncthreads();
+  }
+  const unsigned nfrag = unit_shade<BWD, FROM_HITS, TC, FULL>(it, tb.shells + it.shell0, blockIdx.x, tb.hdr,
+                                                              warp_smem(tb.kmax, BWD, TC), tb.kmax, w, w + 1);
+  if (kBlockCount) {   // one addition to the header per block, by its last warp
+    constexpr unsigned kDone = 1u << 24;   // warps that are through; below, their fragments
+    const unsigned n = __reduce_add_sync(0xffffffffu, nfrag);
+    if ((threadIdx.x & 31) == 0) {
+      const unsigned s = atomicAdd(&s_frags, kDone + n) + kDone + n;
+      if (s / kDone == kWarps && s % kDone) atomicAdd(&tb.hdr->frags, (unsigned long long)(s % kDone));
+    }
+  } else if (!FROM_HITS) {
+    warp_count(&tb.hdr->frags, nfrag);
+  }
 }
 
+// The statistics of a warp of the persistent kernel, counter q of the header.
+constexpr int kCounters = 7;
+__device__ __forceinline__ unsigned long long* counter(WsHeader* h, int q) {
+  return q == 6 ? &h->frags : (q == 5 ? &h->clipped : &h->front + q);
+}
+static_assert(offsetof(WsHeader, large) == offsetof(WsHeader, front) + 32, "front, back, nearc, guard, large");
+
 // Bounded wait (one lane) for `target` completions; false on timeout or
-// abort.  A timeout records VS_ERR_TIMEOUT and raises the abort flag so that
-// every warp leaves the persistent loop.
-static __device__ bool wait_done(const int* ctr, int target, long long limit, WsHeader* hdr) {
+// abort.  A timeout records VS_ERR_TIMEOUT, raises the abort flag, which ends
+// the other waits, and moves the unit counter to the end, so that every warp
+// leaves the persistent loop.
+static __device__ bool wait_done(const int* ctr, int target, long long limit, WsHeader* hdr, int total) {
   for (long long n = 0;; ++n) {
     if (ld_acquire(ctr) >= target) return true;
     if (*(volatile int*)&hdr->abort) return false;
     if (n >= limit) {
       record_error(hdr, VS_ERR_TIMEOUT);
       atomicExch(&hdr->abort, 1);
+      atomicMax(&hdr->next_unit, (unsigned)total);
       return false;
     }
     __nanosleep(200);
@@ -1051,24 +1080,45 @@ static __device__ bool wait_done(const int* ctr, int target, long long limit, Ws
 // stages (while still in L2).  A unit waits only for the previous phase of
 // its own item, whose units were all dispensed in an earlier stage to warps
 // that are already running, so the wait always ends (and is bounded anyway).
+//
+// What a unit costs beside its work is its traffic to single words of the
+// workspace, where the atomics of all warps queue up.  A unit takes one from
+// the header (its number) and one from its item (its completion); the
+// statistics are summed per warp in shared memory and added to the header
+// when the kernel ends, and the abort flag is read by waiting warps only.
 template <bool BWD, int TC, bool FULL>
 __global__ void __launch_bounds__(pers_threads(BWD), BWD ? VS_PERS_BWD_BLOCKS : VS_PERS_FWD_BLOCKS) k_persistent(TableRef tb, long long spin_limit) {
   const unsigned kAll = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   WsHeader* hdr = tb.hdr;
   char* smem = warp_smem(tb.kmax, BWD, TC);
+  // the warp's sums of (front, back, nearc, guard, large, clipped, frags), one
+  // per lane
+  __shared__ unsigned s_count[pers_warps(BWD)][8];
+  unsigned* const my_count = &s_count[threadIdx.x >> 5][lane & 7];
+  if (lane < 8) *my_count = 0;
+  __syncwarp();
+  // adds v (the lane's counter's share of a unit) and passes a sum that
+  // could overflow on to the header
+  auto count = [&](unsigned v) {
+    if (lane < kCounters && v) {
+      const unsigned s = *my_count + v;
+      if (s >= 1u << 31) atomicAdd(counter(hdr, lane), (unsigned long long)s);
+      *my_count = s >= 1u << 31 ? 0 : s;
+    }
+  };
   for (;;) {
-    int g = 0;
-    if (lane == 0) g = *(volatile int*)&hdr->abort ? tb.total : (int)atomicAdd(&hdr->next_unit, 1u);
+    unsigned g = 0;
+    if (lane == 0) g = atomicAdd(&hdr->next_unit, 1u);
     g = __shfl_sync(kAll, g, 0);
-    if (g >= tb.total) break;
+    if (g >= (unsigned)tb.total) break;
     // stage: last s with stage_pre[s] <= g
     int lo = 0, hi = tb.n + NPH - 2;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (__ldg(tb.stage_pre + mid) <= g) lo = mid; else hi = mid - 1;
+      if (__ldg(tb.stage_pre + mid) <= (int)g) lo = mid; else hi = mid - 1;
     }
-    int rel = g - __ldg(tb.stage_pre + lo);
+    int rel = (int)g - __ldg(tb.stage_pre + lo);
     int ph = 0, j = lo;
     for (ph = 0; ph < NPH; ++ph) {
       j = lo - ph;
@@ -1083,7 +1133,7 @@ __global__ void __launch_bounds__(pers_threads(BWD), BWD ? VS_PERS_BWD_BLOCKS : 
       int target = it.units[ph - 1];
       long long lim = spin_limit;
       if (ph == PH_SHADE && it.stall && u == 0) { target += 1; lim = 4096; }
-      ok = wait_done(tb.done + j * NPH + ph - 1, target, lim, hdr) ? 1 : 0;
+      ok = wait_done(tb.done + j * NPH + ph - 1, target, lim, hdr, tb.total) ? 1 : 0;
     }
     ok = __shfl_sync(kAll, ok, 0);
     __syncwarp();   // orders every lane's reads after lane 0's acquire
@@ -1094,17 +1144,19 @@ __global__ void __launch_bounds__(pers_threads(BWD), BWD ? VS_PERS_BWD_BLOCKS : 
       case PH_RASTER: {
         RasterCounts rc = {0, 0, 0, 0};
         unit_raster<FULL>(it, sh, u, smem, rc);
-        warp_count(&hdr->front, rc.fb & 0xFFFFu);
-        warp_count(&hdr->back, rc.fb >> 16);
-        warp_count(&hdr->nearc, rc.ng & 0xFFFFu);
-        warp_count(&hdr->guard, rc.ng >> 16);
-        warp_count(&hdr->large, rc.lc & 0xFFFFu);
-        warp_count(&hdr->clipped, rc.lc >> 16);
+        // a unit's sums are at most its 2048 triangles: both halves stay apart
+        const unsigned fb = __reduce_add_sync(kAll, rc.fb), ng = __reduce_add_sync(kAll, rc.ng),
+                       lc = __reduce_add_sync(kAll, rc.lc);
+        const unsigned pair = lane < 2 ? fb : (lane < 4 ? ng : lc);
+        count(lane < 6 ? (lane & 1 ? pair >> 16 : pair & 0xFFFFu) : 0);
         if (__any_sync(kAll, rc.bad) && lane == 0) record_error(hdr, VS_ERR_INVALID_ARG);
         break;
       }
-      default:
-        unit_shade<BWD, false, TC, FULL>(it, sh, u, hdr, smem, tb.kmax, 0, it.shade_rounds);
+      default: {
+        const unsigned n = unit_shade<BWD, false, TC, FULL>(it, sh, u, hdr, smem, tb.kmax, 0, it.shade_rounds);
+        const unsigned frags = __reduce_add_sync(kAll, n);
+        count(lane == 6 ? frags : 0);
+      }
     }
     __syncwarp();
     if (lane == 0) {
@@ -1112,6 +1164,7 @@ __global__ void __launch_bounds__(pers_threads(BWD), BWD ? VS_PERS_BWD_BLOCKS : 
       atomicAdd(tb.done + j * NPH + ph, 1);
     }
   }
+  if (lane < kCounters && *my_count) atomicAdd(counter(hdr, lane), (unsigned long long)*my_count);
 }
 
 }  // namespace vsd

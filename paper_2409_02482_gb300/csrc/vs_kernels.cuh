@@ -1060,7 +1060,7 @@ static_assert(offsetof(WsHeader, large) == offsetof(WsHeader, front) + 32, "fron
 // leaves the persistent loop.
 static __device__ bool wait_done(const int* ctr, int target, long long limit, WsHeader* hdr, int total) {
   for (long long n = 0;; ++n) {
-    if (ld_acquire(ctr) >= target) return true;
+    if (ld_relaxed(ctr) >= target) return ld_acquire(ctr) >= target;
     if (*(volatile int*)&hdr->abort) return false;
     if (n >= limit) {
       record_error(hdr, VS_ERR_TIMEOUT);
@@ -1086,6 +1086,14 @@ static __device__ bool wait_done(const int* ctr, int target, long long limit, Ws
 // the header (its number) and one from its item (its completion); the
 // statistics are summed per warp in shared memory and added to the header
 // when the kernel ends, and the abort flag is read by waiting warps only.
+//
+// A fence or an acquire at GPU scope also empties the SM's L1, on which every
+// fragment's chain of index, vertex and UV loads depends.  So a unit's
+// completion is a release reduction and no fence, a wait polls with relaxed
+// loads, and a phase that one warp of the block has acquired is taken by the
+// others from shared memory: an acquire per block, item and phase instead of
+// one per unit and poll (fitting step of 24 views at 800^2: 8.83 -> 8.42 ms;
+// 32 views forward 4.66 -> 4.51 ms).
 template <bool BWD, int TC, bool FULL>
 __global__ void __launch_bounds__(pers_threads(BWD), BWD ? VS_PERS_BWD_BLOCKS : VS_PERS_FWD_BLOCKS) k_persistent(TableRef tb, long long spin_limit) {
   const unsigned kAll = 0xffffffffu;
@@ -1097,7 +1105,11 @@ __global__ void __launch_bounds__(pers_threads(BWD), BWD ? VS_PERS_BWD_BLOCKS : 
   __shared__ unsigned s_count[pers_warps(BWD)][8];
   unsigned* const my_count = &s_count[threadIdx.x >> 5][lane & 7];
   if (lane < 8) *my_count = 0;
-  __syncwarp();
+  // the item whose phase (setup, raster) a warp of this block last saw done,
+  // by item modulo 4
+  __shared__ int s_seen[NPH - 1][4];
+  if (threadIdx.x < (NPH - 1) * 4) (&s_seen[0][0])[threadIdx.x] = -1;
+  __syncthreads();
   // adds v (the lane's counter's share of a unit) and passes a sum that
   // could overflow on to the header
   auto count = [&](unsigned v) {
@@ -1132,8 +1144,13 @@ __global__ void __launch_bounds__(pers_threads(BWD), BWD ? VS_PERS_BWD_BLOCKS : 
     if (lane == 0 && ph > 0) {
       int target = it.units[ph - 1];
       long long lim = spin_limit;
-      if (ph == PH_SHADE && it.stall && u == 0) { target += 1; lim = 4096; }
-      ok = wait_done(tb.done + j * NPH + ph - 1, target, lim, hdr, tb.total) ? 1 : 0;
+      int* seen = &s_seen[ph - 1][j & 3];
+      const bool stall = ph == PH_SHADE && it.stall && u == 0;
+      if (stall) { target += 1; lim = 4096; }
+      if (stall || ld_acquire_shared(seen) != j) {
+        ok = wait_done(tb.done + j * NPH + ph - 1, target, lim, hdr, tb.total) ? 1 : 0;
+        if (ok) st_release_shared(seen, j);
+      }
     }
     ok = __shfl_sync(kAll, ok, 0);
     __syncwarp();   // orders every lane's reads after lane 0's acquire
@@ -1159,10 +1176,7 @@ __global__ void __launch_bounds__(pers_threads(BWD), BWD ? VS_PERS_BWD_BLOCKS : 
       }
     }
     __syncwarp();
-    if (lane == 0) {
-      __threadfence();
-      atomicAdd(tb.done + j * NPH + ph, 1);
-    }
+    if (lane == 0) red_release_add(tb.done + j * NPH + ph, 1);   // after the whole warp's writes
   }
   if (lane < kCounters && *my_count) atomicAdd(counter(hdr, lane), (unsigned long long)*my_count);
 }

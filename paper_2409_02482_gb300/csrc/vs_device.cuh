@@ -130,7 +130,8 @@ struct alignas(16) DShell {
   int32_t vec;                 // texel load width in values (1, 2, 4, 8)
   int32_t gvec;                // gradient atomic width in floats (1, 2, 4)
   int32_t wide;                // texels 32-byte aligned (base and pitch): 256-bit loads
-  int4* pad5;                  // unused
+  int32_t raster_tris;         // triangles per raster unit (a power of two)
+  int32_t pad5;
   // VS_TEX_SH_U8: byte offset of band l in tex, resolution shift per band,
   // decode value = vmin + vscale * q
   long long boff[4];
@@ -149,7 +150,6 @@ struct alignas(16) DItem {
   float* layers;               // [k, H*W, 12] per-layer buffers or null
   int32_t k, shell0, raster_lg, clear_units;   // raster_lg: a unit of one triangle is shared by 2^raster_lg units
   int32_t flags, do_bwd, stall;
-  int32_t raster_tris;         // triangles per raster unit (a power of two)
   int32_t shade_rounds;        // shading unit = 32 * shade_rounds pixels
   int32_t setup_verts;         // vertices per setup unit
   int32_t clear_words;         // visibility words per clearing unit (even)

@@ -309,7 +309,7 @@ __device__ __forceinline__ void raster_round(const DItem& it, const DShell& s, i
   __syncwarp();   // the records are reused by the next round
 }
 
-// Raster unit u: it.raster_tris consecutive triangles of one shell in rounds
+// Raster unit u: s.raster_tris consecutive triangles of one shell in rounds
 // of 32 (or one triangle shared by 2^raster_lg units).  The next round's
 // indices are loaded while the current one runs.
 template <bool FULL>
@@ -320,8 +320,8 @@ static __device__ __forceinline__ void unit_raster(const DItem& it, const DShell
   int i = 0;
   while (i + 1 < it.k && u >= it.raster_pre[i + 1]) ++i;
   const DShell& s = sh[i];
-  const int base = (u - it.raster_pre[i]) * it.raster_tris;
-  const int end = min(s.nt, base + it.raster_tris);
+  const int base = (u - it.raster_pre[i]) * s.raster_tris;
+  const int end = min(s.nt, base + s.raster_tris);
   unsigned long long* vis = it.vis + (size_t)i * it.cam.W * it.cam.H;
   const int lane = threadIdx.x & 31;
   int3 ix = load_index(s, base + lane);

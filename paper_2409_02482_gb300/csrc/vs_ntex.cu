@@ -857,10 +857,11 @@ int fused_forward_tc(const vs_ntex_config& c, const Views& P, const Enc& e, int 
   int dev = 0, sms = 0;
   VS_TRY_CUDA(cudaGetDevice(&dev));
   VS_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  // two CTAs per SM at most: 2 x 256 tensor-memory columns, and the shared
-  // memory of a third would not fit
-  const int per_sm = 2 * (smem + 1024) <= 228 * 1024 ? 2 : 1;
-  MlpFwdArgs a{P.table, P.W0, P.b0, P.W1, P.b1, P.W2, P.b2, texels, W, H, W * H, c.out_ch, LF, dtype, pitch, ch0,
+  // as many CTAs per SM as fit its shared memory and registers (their 3 x 128
+  // tensor-memory columns always do)
+  const int per_sm = 3 * (smem + 1024) <= 228 * 1024 ? 3 : 2;
+  const int vec = pitch % 4 == 0 && ch0 % 4 == 0 && (uintptr_t)texels % (dtype == 1 ? 8 : 16) == 0;
+  MlpFwdArgs a{P.table, P.W0, P.b0, P.W1, P.b1, P.W2, P.b2, texels, W, H, W * H, c.out_ch, LF, dtype, pitch, ch0, vec,
                status, 1ll << 22};
   k_mlp_fwd_tc<<<sms * per_sm, kFwdThreads, smem, st>>>(a, e);
   return (int)cudaGetLastError();
@@ -987,11 +988,12 @@ int fused_backward_tc(const vs_ntex_config& c, const Views& P, float* const g[7]
   const int rows_ws = N < kNtexChunk ? N : kNtexChunk;
   const int chunk = N < 4 * rows_ws ? N : 4 * rows_ws;
   const Ws w = carve(c, 1, ws);
+  const int vec = pitch % 4 == 0 && ch0 % 4 == 0 && (uintptr_t)grad % 16 == 0;
   float* dX = reinterpret_cast<float*>(ws) + 64;
   for (int n0 = 0; n0 < N; n0 += chunk) {
     const int count = N - n0 < chunk ? N - n0 : chunk;
     MlpBwdArgs a{P.table, P.W0, P.b0, P.W1, P.b1, P.W2, grad, g[1], g[2], g[3], g[4], g[5], g[6], dX,
-                 W, H, n0, count, c.out_ch, LF, c.features, pitch, ch0, w.status, 1ll << 22};
+                 W, H, n0, count, c.out_ch, LF, c.features, pitch, ch0, vec, w.status, 1ll << 22};
     k_mlp_bwd_tc<<<sms, kBwdThreads, smem, st>>>(a, e);   // one CTA per SM (shared memory)
     VS_TRY_CUDA(cudaGetLastError());
     VS_TRY(table_grad(e, dX, (long long)count * c.features, c.features, W, H, n0, count, g[0], st));

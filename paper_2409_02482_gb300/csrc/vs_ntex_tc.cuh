@@ -228,6 +228,7 @@ struct MlpFwdArgs {
   const float *table, *W0, *b0, *W1, *b1, *W2, *b2;
   void* texels;
   int W, H, N, C, LF, dtype, pitch, ch0;
+  int vec;   // 4 consecutive channels can be stored at once
   int* status;
   long long spin_limit;
 };
@@ -251,12 +252,15 @@ __device__ __forceinline__ void stage_op(float* dst, const float* src, int n_row
   }
 }
 
-// Encoding of texel (tx, ty), levels [l0, l1), into row m of the canonical
-// operand X (TF32).  With two features per level the levels go four at a
+// Encoding of texel n, levels [l0, l1), into row m of the canonical operand X
+// (TF32; zeros unless live, n then any texel).  Every lane of the warp takes
+// part, with the same levels (WarpCorners).  With two features per level the levels go four at a
 // time, all sixteen corner rows (8 bytes each) loaded before any is used;
 // the sums run in the same order as the generic loop.
-__device__ __forceinline__ void encode_row(const Enc& e, const float* table, int tx, int ty, int W, int H, int l0,
+__device__ __forceinline__ void encode_row(const Enc& e, const float* table, int n, bool live, int W, int H, int l0,
                                            int l1, float* X, int m, int Kp) {
+  const int ty = n / W, tx = n - ty * W;
+  const WarpCorners wc(e, ty, H);
   if (e.F == 2) {
     const float2* t2 = reinterpret_cast<const float2*>(table);
     for (int lb = l0; lb < l1; lb += 4) {
@@ -267,7 +271,7 @@ __device__ __forceinline__ void encode_row(const Enc& e, const float* table, int
         const int l = lb + d < l1 ? lb + d : lb;
         const size_t lt = (size_t)l << e.logT;
         uint32_t row[4];
-        corners4(e, l, tx, ty, W, H, row, w[d]);
+        wc.at(e, l, tx, ty, W, H, row, w[d]);
 #pragma unroll
         for (int c = 0; c < 4; ++c) v[d][c] = __ldg(t2 + lt + row[c]);
       }
@@ -280,8 +284,8 @@ __device__ __forceinline__ void encode_row(const Enc& e, const float* table, int
             a0 = fmaf(w[d][c], v[d][c].x, a0);
             a1 = fmaf(w[d][c], v[d][c].y, a1);
           }
-          *op_at(X, m, 2 * (lb + d), Kp) = tf32_rna(a0);
-          *op_at(X, m, 2 * (lb + d) + 1, Kp) = tf32_rna(a1);
+          *reinterpret_cast<float2*>(op_at(X, m, 2 * (lb + d), Kp)) =
+              live ? make_float2(tf32_rna(a0), tf32_rna(a1)) : make_float2(0.0f, 0.0f);
         }
       }
     }
@@ -292,12 +296,12 @@ __device__ __forceinline__ void encode_row(const Enc& e, const float* table, int
     const size_t lt = (size_t)l << e.logT;
     uint32_t row[4];
     float w[4];
-    corners4(e, l, tx, ty, W, H, row, w);
+    wc.at(e, l, tx, ty, W, H, row, w);
     for (int c = 0; c < 4; ++c) {
       const float* t = table + (lt + row[c]) * e.F;
       for (int f = 0; f < e.F; ++f) acc[f] = fmaf(w[c], __ldg(t + f), acc[f]);
     }
-    for (int f = 0; f < e.F; ++f) *op_at(X, m, l * e.F + f, Kp) = tf32_rna(acc[f]);
+    for (int f = 0; f < e.F; ++f) *op_at(X, m, l * e.F + f, Kp) = live ? tf32_rna(acc[f]) : 0.0f;
   }
 }
 
@@ -351,7 +355,8 @@ __device__ __forceinline__ bool wait_mma(uint64_t* bar, uint32_t& phase, int* st
   return ok;
 }
 
-constexpr int kMlpTmemCols = 256;   // D0 [0, 64), D1 [64, 128), D2 [128, 128 + Cp)
+constexpr int kMlpTmemCols = 256;   // the adjoint's: D0 [0, 64), D1 [64, 128), D2 [128, 192)
+constexpr int kFwdTmemCols = 128;   // the forward's: both hidden layers [0, 64), outputs [64, 64 + Cp)
 
 // Four consecutive values k .. k + 3 (k % 4 == 0) of row m: one 16-byte
 // access (a warp's 32 rows then cover 512 contiguous-in-groups bytes:
@@ -368,31 +373,35 @@ __device__ __forceinline__ float4 relu_tf32(const float* v, const float* b, bool
 
 // Dynamic shared memory of k_mlp_fwd_tc for LF inputs and C outputs.
 __host__ __device__ constexpr int mlp_fwd_smem(int LF, int C) {
-  return op_bytes(kMlpH, LF) + op_bytes(kMlpH, kMlpH) + op_bytes((C + 15) & ~15, kMlpH) + op_bytes(128, LF) +
-         2 * op_bytes(128, kMlpH) + 256;
+  return op_bytes(kMlpH, LF) + op_bytes(kMlpH, kMlpH) + op_bytes((C + 15) & ~15, kMlpH) + op_bytes(128, kMlpH) + 256;
 }
 
-// 8 warps per CTA, as in the adjoint: warps w and w + 4 share a tensor-memory
-// lane quarter (texel rows) and split the columns and the encoding's levels.
+// 8 warps per CTA: warps w and w + 4 share a tensor-memory lane quarter (texel
+// rows) and split the columns and the encoding's levels.  What bounds the
+// kernel is the latency of the encoding's gathers and of the chain of
+// products (tensor pipe 5 % active), so it wants CTAs: a tile's activations
+// share one 32 KB buffer, each layer's outputs over its inputs, and three
+// CTAs fit an SM instead of two (16 x 2 -> 64 -> 64 -> 27 network at 2048^2,
+// forward and adjoint: 5.59 -> 5.33 ms).
 constexpr int kFwdThreads = 256;
 
-__global__ void __launch_bounds__(kFwdThreads, 2) k_mlp_fwd_tc(const MlpFwdArgs a, const __grid_constant__ Enc e) {
+__global__ void __launch_bounds__(kFwdThreads, 3) k_mlp_fwd_tc(const MlpFwdArgs a, const __grid_constant__ Enc e) {
   extern __shared__ __align__(128) char msm[];
   const int LFp = (a.LF + 7) & ~7, Cp = (a.C + 15) & ~15;
   float* W0s = reinterpret_cast<float*>(msm);
   float* W1s = W0s + kMlpH * LFp;
   float* W2s = W1s + kMlpH * kMlpH;
   float* Xs = W2s + Cp * kMlpH;
-  float* H1s = Xs + 128 * LFp;
-  float* H2s = H1s + 128 * kMlpH;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(H2s + 128 * kMlpH);
+  float* const H1s = Xs;   // each layer's outputs take the place of its inputs:
+  float* const H2s = Xs;   // every thread has waited for the MMAs that read them
+  uint64_t* bar = reinterpret_cast<uint64_t*>(Xs + 128 * kMlpH);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 1);
   const int tid = threadIdx.x, warp = tid >> 5;
   const int half = tid >> 7, r = tid & 127;        // column half, texel row of the tile
   const int l_lo = half ? (e.L + 1) / 2 : 0, l_hi = half ? e.L : (e.L + 1) / 2;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(kMlpTmemCols)
+                 "r"(kFwdTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -414,9 +423,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) k_mlp_fwd_tc(const MlpFwdArgs 
   for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     // encoding of texel n = 128 tile + r into row r of X (this half's levels)
     const int n = tile * 128 + r;
-    if (n < a.N) encode_row(e, a.table, n % a.W, n / a.W, a.W, a.H, l_lo, l_hi, Xs, r, LFp);
-    else
-      for (int k = l_lo * e.F; k < l_hi * e.F; ++k) *op_at(Xs, r, k, LFp) = 0.0f;
+    encode_row(e, a.table, min(n, a.N - 1), n < a.N, a.W, a.H, l_lo, l_hi, Xs, r, LFp);
     if (half == 0)
       for (int k = a.LF; k < LFp; ++k) *op_at(Xs, r, k, LFp) = 0.0f;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -438,11 +445,11 @@ __global__ void __launch_bounds__(kFwdThreads, 2) k_mlp_fwd_tc(const MlpFwdArgs 
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     // layer 1
-    if (tid == 0) mma_tile(tmem + 64u, H1s, W1s, kMlpH, kMlpH, bar);
+    if (tid == 0) mma_tile(tmem, H1s, W1s, kMlpH, kMlpH, bar);
     ok = wait_mma(bar, phase, a.status, a.spin_limit) && ok;
     for (int c0 = 32 * half; c0 < 32 * half + 32; c0 += 16) {
       float v[16];
-      tmem_ld16(tmem + lane_base + 64u + (uint32_t)c0, v);
+      tmem_ld16(tmem + lane_base + (uint32_t)c0, v);
 #pragma unroll
       for (int j = 0; j < 16; j += 4)
         st4(H2s, r, c0 + j, kMlpH, relu_tf32(v + j, a.b1 + c0 + j, true));
@@ -452,20 +459,34 @@ __global__ void __launch_bounds__(kFwdThreads, 2) k_mlp_fwd_tc(const MlpFwdArgs 
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     // output layer -> texels
-    if (tid == 0) mma_tile(tmem + 128u, H2s, W2s, kMlpH, Cp, bar);
+    if (tid == 0) mma_tile(tmem + 64u, H2s, W2s, kMlpH, Cp, bar);
     ok = wait_mma(bar, phase, a.status, a.spin_limit) && ok;
     for (int c0 = 16 * half; c0 < Cp; c0 += 32) {
       float v[16];
-      tmem_ld16(tmem + lane_base + 128u + (uint32_t)c0, v);
+      tmem_ld16(tmem + lane_base + 64u + (uint32_t)c0, v);
       if (n < a.N) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int c = c0 + j;
-          if (c >= a.C) break;
-          const float y = ok ? v[j] + __ldg(a.b2 + c) : 0.0f;
-          const size_t off = (size_t)n * a.pitch + a.ch0 + c;
-          if (a.dtype == 1) reinterpret_cast<__half*>(a.texels)[off] = __float2half_rn(y);
-          else reinterpret_cast<float*>(a.texels)[off] = y;
+        for (int j = 0; j < 16; ++j) v[j] = ok && c0 + j < a.C ? v[j] + __ldg(a.b2 + c0 + j) : 0.0f;
+        const size_t off = (size_t)n * a.pitch + a.ch0 + c0;
+#pragma unroll
+        for (int j = 0; j < 16; j += 4) {
+          if (a.vec && c0 + j + 4 <= a.C) {
+            if (a.dtype == 1) {
+              const __half2 h0 = __floats2half2_rn(v[j], v[j + 1]), h1 = __floats2half2_rn(v[j + 2], v[j + 3]);
+              *reinterpret_cast<uint2*>(reinterpret_cast<__half*>(a.texels) + off + j) =
+                  make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+            } else {
+              *reinterpret_cast<float4*>(reinterpret_cast<float*>(a.texels) + off + j) =
+                  make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+            }
+          } else {
+#pragma unroll
+            for (int d = j; d < j + 4; ++d) {
+              if (c0 + d >= a.C) break;
+              if (a.dtype == 1) reinterpret_cast<__half*>(a.texels)[off + d] = __float2half_rn(v[d]);
+              else reinterpret_cast<float*>(a.texels)[off + d] = v[d];
+            }
+          }
         }
       }
     }
@@ -476,7 +497,7 @@ __global__ void __launch_bounds__(kFwdThreads, 2) k_mlp_fwd_tc(const MlpFwdArgs 
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kMlpTmemCols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kFwdTmemCols) : "memory");
 }
 
 }  // namespace vsn
@@ -500,6 +521,7 @@ struct MlpBwdArgs {
   float *dW0, *db0, *dW1, *db1, *dW2, *db2;
   float* dX;           // dL/d(encoding) of texels n0 .. n0 + count, level-major [L][count][F]
   int W, H, n0, count, C, LF, F, pitch, ch0;
+  int vec;             // 4 consecutive channels of grad can be loaded at once
   int* status;
   long long spin_limit;
 };
@@ -636,23 +658,44 @@ __global__ void __launch_bounds__(kBwdThreads, 1) k_mlp_bwd_tc(const MlpBwdArgs 
   for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const int i = tile * 128 + r, n = a.n0 + i;
     const bool live = i < a.count;
-    const int tx = live ? n % a.W : 0, ty = live ? n / a.W : 0;
     // encoding of row r (this group's levels) and the output gradient (this
     // group's columns)
-    if (live) encode_row(e, a.table, tx, ty, a.W, a.H, l_lo, l_hi, Xs, r, LFp);
-    else
-      for (int k = l_lo * e.F; k < l_hi * e.F; ++k) *op_at(Xs, r, k, LFp) = 0.0f;
+    encode_row(e, a.table, live ? n : a.n0 + a.count - 1, live, a.W, a.H, l_lo, l_hi, Xs, r, LFp);
     if (quad == 0)
       for (int k = LF; k < LFp; ++k) *op_at(Xs, r, k, LFp) = 0.0f;
     // dY kept in FP32 (the tensor cores read its TF32 part; the bias and
     // weight gradients of the output layer use all of it)
+    const float* src = a.grad + (size_t)n * a.pitch + a.ch0;
+    if (a.vec && (Cp / NG) % 4 == 0) {
 #pragma unroll
-    for (int q = 0; q < kDy; ++q) {
-      const int c = quad * (Cp / NG) + q;
-      if (q < Cp / NG) {
-        const float v = (live && c < a.C) ? __ldg(a.grad + (size_t)n * a.pitch + a.ch0 + c) : 0.0f;
-        *op_at(dYs, r, c, Cp) = v;
-        gb2[q] += v;
+      for (int q = 0; q < kDy; q += 4) {
+        const int c = quad * (Cp / NG) + q;
+        if (q < Cp / NG) {
+          float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (live && c < a.C) {
+            if (c + 4 <= a.C) v = __ldg(reinterpret_cast<const float4*>(src + c));
+            else {
+              v.x = __ldg(src + c);
+              if (c + 1 < a.C) v.y = __ldg(src + c + 1);
+              if (c + 2 < a.C) v.z = __ldg(src + c + 2);
+            }
+          }
+          st4(dYs, r, c, Cp, v);
+          gb2[q] += v.x;
+          gb2[q + 1] += v.y;
+          gb2[q + 2] += v.z;
+          gb2[q + 3] += v.w;
+        }
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < kDy; ++q) {
+        const int c = quad * (Cp / NG) + q;
+        if (q < Cp / NG) {
+          const float v = (live && c < a.C) ? __ldg(src + c) : 0.0f;
+          *op_at(dYs, r, c, Cp) = v;
+          gb2[q] += v;
+        }
       }
     }
     sync_for_mma();
@@ -737,7 +780,13 @@ __global__ void __launch_bounds__(kBwdThreads, 1) k_mlp_bwd_tc(const MlpBwdArgs 
     for (int c0 = 16 * quad; c0 < LF16; c0 += 16 * NG) {
       float v[16];
       tmem_ld16(tmem + lane_base + 64u + (uint32_t)c0, v);
-      if (live) {
+      if (live && a.F == 2) {   // a level's two features: 8 bytes, texels contiguous
+#pragma unroll
+        for (int j = 0; j < 16; j += 2)
+          if (c0 + j < LF)
+            *reinterpret_cast<float2*>(a.dX + ((size_t)((c0 + j) >> 1) * a.count + i) * 2) =
+                ok ? make_float2(v[j], v[j + 1]) : make_float2(0.0f, 0.0f);
+      } else if (live) {
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
           if (c0 + j < LF) {

@@ -377,3 +377,42 @@ def test_adam_vector_and_scalar_parameters(vs, ctx, n, shift):
         got = b.cpu().numpy()
         assert np.abs(got[shift:shift + n] - r).max() <= 1e-5
         assert np.all(got[:shift] == 9.0) and np.all(got[shift + n:] == 9.0)
+
+
+@pytest.mark.parametrize("levels,features,out_ch,W,H,pad,ch0", [
+    (3, 1, 1, 129, 31, 1, 0),        # 3 encoding values, one output, scalar channels
+    (16, 2, 27, 2100, 2, 5, 0),      # rows of 2100 texels: tiles within one row
+    (16, 2, 32, 127, 33, 0, 4),      # aligned channels, outputs to the brim
+    (8, 4, 30, 130, 32, 2, 2),       # channels off their 16-byte alignment
+    (4, 4, 9, 16, 260, 3, 0),        # rows shorter than a warp
+])
+def test_ntex_tensor_core_shapes_match_oracle(vs, ctx, levels, features, out_ch, W, H, pad, ch0):
+    """The fused TF32 kernels at the edges of their tiles, channel vectors and
+    encoding, texels and gradients within the TF32 bars of
+    test_ntex_tensor_core_mode_is_close, other channels left alone."""
+    cfg = ntex.NtexConfig(levels=levels, features=features, log2_table=10, base_res=4, growth=1.25, hidden=64,
+                          out_ch=out_ch)
+    params = _params(cfg, 200 + out_ch)
+    nt = vs.NeuralTexture(ctx, cfg.levels, cfg.features, cfg.log2_table, cfg.base_res, cfg.growth, cfg.hidden,
+                          cfg.out_ch, tex_w=W, tex_h=H, tensor_cores=True)
+    nt.params.copy_(torch.from_numpy(params))
+    pitch = out_ch + ch0 + pad
+    ref = ntex.forward(cfg, params.astype(np.float64), W, H)[0].reshape(H, W, out_ch)
+    for dtype in (torch.float32, torch.float16):
+        tex = torch.full((H, W, pitch), 7.0, device="cuda", dtype=dtype)
+        nt.forward(tex, ch0=ch0)
+        got = tex.double().cpu().numpy()
+        assert np.linalg.norm(got[..., ch0:ch0 + out_ch] - ref) <= 2e-3 * np.linalg.norm(ref)
+        assert np.all(got[..., :ch0] == 7.0) and np.all(got[..., ch0 + out_ch:] == 7.0)
+    g = torch.randn((H, W, pitch), device="cuda", generator=torch.Generator("cuda").manual_seed(14))
+    nt.backward(g, ch0=ch0)
+    rg = ntex.backward(cfg, params.astype(np.float64), W, H,
+                       g.cpu().numpy()[..., ch0:ch0 + out_ch].astype(np.float64))
+    q = nt.grads.cpu().numpy().astype(np.float64)
+    lay, _ = cfg.layout()
+    for name, off, shp in lay:
+        n = int(np.prod(shp))
+        bar = 1e-5 if name == "b2" else 8e-2
+        r = rg[off:off + n]
+        assert np.linalg.norm(q[off:off + n] - r) <= bar * np.linalg.norm(r) + 1e-30, name
+    assert nt.status() == 0

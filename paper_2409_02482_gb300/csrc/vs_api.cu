@@ -107,7 +107,7 @@ vs_status baked_layout(int32_t tw, int32_t th, int32_t degree, int32_t shift, Ba
   return VS_OK;
 }
 
-size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 int gcd_pow2(uint64_t a, int cap) {  // largest power of two <= cap dividing a
   int g = 1;
@@ -501,30 +501,67 @@ size_t upload_chunks(const Plan& P) {
   return std::max<size_t>(1, (bytes + kUploadBytes - 1) / kUploadBytes);
 }
 
+// The table's bytes (zero-filled gaps and completion counters).
+void fill_table(const Plan& P, char* dst) {
+  std::memset(dst, 0, P.table_end - P.off_items);
+  std::memcpy(dst, P.items.data(), sizeof(DItem) * P.items.size());
+  std::memcpy(dst + (P.off_shells - P.off_items), P.shells.data(), sizeof(DShell) * P.shells.size());
+  std::memcpy(dst + (P.off_stage - P.off_items), P.stage_pre.data(), sizeof(int) * P.stage_pre.size());
+}
+
+template <int BYTES>
+void fill_chunk(const Plan& P, Upload<BYTES>& c, size_t pos, size_t nb, bool first, int launches) {
+  c.dst_off = (uint32_t)(P.off_items + pos);
+  c.nbytes = (uint32_t)nb;
+  c.reset = first ? 1 : 0;
+  c.launches = launches;
+  c.kernel_class = 1 + P.tc + (P.full ? 16 : 0);
+}
+
 // Copies the table (items, shells, zeroed completion counters, stage
 // prefixes) into the workspace through kernel parameters; `kernels` is the
 // number of compute kernels the call enqueues after the upload.
 vs_status upload_table(const Plan& P, char* ws, int kernels, cudaStream_t st) {
   std::vector<char> blob(P.table_end - P.off_items, 0);
-  std::memcpy(blob.data(), P.items.data(), sizeof(DItem) * P.items.size());
-  std::memcpy(blob.data() + (P.off_shells - P.off_items), P.shells.data(), sizeof(DShell) * P.shells.size());
-  std::memcpy(blob.data() + (P.off_stage - P.off_items), P.stage_pre.data(), sizeof(int) * P.stage_pre.size());
+  fill_table(P, blob.data());
   static thread_local UploadChunk chunk;
+  static thread_local SmallUpload small;
   const size_t nchunks = upload_chunks(P);
   size_t pos = 0;
   for (size_t c = 0; c < nchunks; ++c) {
     const size_t nb = std::min(blob.size() - pos, (size_t)kUploadBytes);
-    chunk.dst_off = (uint32_t)(P.off_items + pos);
-    chunk.nbytes = (uint32_t)nb;
-    chunk.reset = c == 0 ? 1 : 0;
-    chunk.launches = c == 0 ? (int32_t)(nchunks + kernels) : 0;
-    chunk.kernel_class = 1 + P.tc + (P.full ? 16 : 0);
-    std::memcpy(chunk.data, blob.data() + pos, nb);
-    cudaError_t e = vsk::upload(ws, chunk, st);
+    const int launches = c == 0 ? (int)nchunks + kernels : 0;
+    cudaError_t e;
+    if (nb <= (size_t)kSmallUploadBytes) {
+      fill_chunk(P, small, pos, nb, c == 0, launches);
+      std::memcpy(small.data, blob.data() + pos, nb);
+      e = vsk::upload(ws, small, st);
+    } else {
+      fill_chunk(P, chunk, pos, nb, c == 0, launches);
+      std::memcpy(chunk.data, blob.data() + pos, nb);
+      e = vsk::upload(ws, chunk, st);
+    }
     if (e != cudaSuccess) return cuda_fail(e, "table upload launch");
     pos += nb;
   }
   return VS_OK;
+}
+
+// The table of a single view, for its setup kernel's parameters.
+static_assert(align256(sizeof(DItem)) + align256(sizeof(DShell) * kMaxShells) + 1024 <= kSmallUploadBytes,
+              "a single view's table fits the parameters");
+const SmallUpload& plain_table(const Plan& P, int kernels) {
+  static thread_local SmallUpload t;
+  const size_t nb = P.table_end - P.off_items;
+  fill_chunk(P, t, 0, nb, true, kernels);
+  fill_table(P, reinterpret_cast<char*>(t.data));
+  return t;
+}
+
+cudaError_t run_plain_forward(const vs_ctx* ctx, const Plan& P, char* ws, cudaStream_t st) {
+  const int* units = P.items[0].units;
+  return vsk::plain_forward(table_ref(P, ws), ws, plain_table(P, vsk::plain_forward_launches(units)),
+                            (uint32_t)(P.off_shells - P.off_items), units, P.tc, P.full, ctx->num_sms, st);
 }
 
 vs_status check_ws(const Plan& P, void* ws, size_t ws_bytes) {
@@ -828,8 +865,7 @@ vs_status vs_render(vs_ctx* ctx, const vs_object* obj, const vs_camera* cam, con
   if ((s = make_plan(&r, 1, bg, 0, true, flags & ~VS_FLAG_TEST_STALL, ws, P, plain_shape(ctx))) != VS_OK) return s;
   if ((s = check_ws(P, workspace, ws_bytes)) != VS_OK) return s;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if ((s = upload_table(P, ws, vsk::plain_forward_launches(P.items[0].units), st)) != VS_OK) return s;
-  cudaError_t e = vsk::plain_forward(table_ref(P, ws), P.items[0].units, P.tc, P.full, ctx->num_sms, st);
+  cudaError_t e = run_plain_forward(ctx, P, ws, st);
   return e == cudaSuccess ? VS_OK : cuda_fail(e, "vs_render launch");
 }
 
@@ -850,8 +886,7 @@ vs_status vs_render_layers(vs_ctx* ctx, const vs_object* obj, const vs_camera* c
   if ((s = make_plan(&r, 1, bg, 0, true, flags & ~VS_FLAG_TEST_STALL, ws, P, plain_shape(ctx))) != VS_OK) return s;
   if ((s = check_ws(P, workspace, ws_bytes)) != VS_OK) return s;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if ((s = upload_table(P, ws, vsk::plain_forward_launches(P.items[0].units), st)) != VS_OK) return s;
-  cudaError_t e = vsk::plain_forward(table_ref(P, ws), P.items[0].units, P.tc, P.full, ctx->num_sms, st);
+  cudaError_t e = run_plain_forward(ctx, P, ws, st);
   return e == cudaSuccess ? VS_OK : cuda_fail(e, "vs_render_layers launch");
 }
 
@@ -875,8 +910,9 @@ vs_status vs_render_backward(vs_ctx* ctx, const vs_object* obj, const vs_camera*
   if ((s = make_plan(&r, 1, bg, 1, false, flags & ~VS_FLAG_TEST_STALL, ws, P, plain_shape(ctx))) != VS_OK) return s;
   if ((s = check_ws(P, workspace, ws_bytes)) != VS_OK) return s;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if ((s = upload_table(P, ws, vsk::plain_backward_launches(P.items[0].units), st)) != VS_OK) return s;
-  cudaError_t e = vsk::plain_backward(table_ref(P, ws), P.items[0].units, P.tc, P.full, st);
+  const int* units = P.items[0].units;
+  cudaError_t e = vsk::plain_backward(table_ref(P, ws), ws, plain_table(P, vsk::plain_backward_launches(units)),
+                                      (uint32_t)(P.off_shells - P.off_items), units, P.tc, P.full, st);
   return e == cudaSuccess ? VS_OK : cuda_fail(e, "vs_render_backward launch");
 }
 
@@ -1274,7 +1310,6 @@ extern "C" vs_status vs_render_noalloc(vs_ctx* ctx, const vs_object* obj, const 
   // cleared by the setup kernel and the table is rewritten below
   cudaError_t e = cudaMemsetAsync(ws, 0, sizeof(WsHeader), st);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(no-alloc header)");
-  if ((s = upload_table(P, ws, vsk::plain_forward_launches(P.items[0].units), st)) != VS_OK) return s;
-  e = vsk::plain_forward(table_ref(P, ws), P.items[0].units, P.tc, P.full, ctx->num_sms, st);
+  e = run_plain_forward(ctx, P, ws, st);
   return e == cudaSuccess ? VS_OK : cuda_fail(e, "vs_render_noalloc launch");
 }

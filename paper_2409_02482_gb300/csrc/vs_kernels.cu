@@ -6,7 +6,8 @@
 
 namespace vsd {
 
-__global__ void __launch_bounds__(kThreads) k_upload(char* ws, const __grid_constant__ UploadChunk c) {
+template <int BYTES>
+__device__ __forceinline__ void write_chunk(char* ws, const Upload<BYTES>& c) {
   uint4* dst = reinterpret_cast<uint4*>(ws + c.dst_off);
   for (uint32_t i = threadIdx.x; i < c.nbytes / 16; i += blockDim.x) dst[i] = c.data[i];
   if (c.reset && threadIdx.x == 0) {
@@ -18,13 +19,27 @@ __global__ void __launch_bounds__(kThreads) k_upload(char* ws, const __grid_cons
   }
 }
 
+template <int BYTES>
+__global__ void __launch_bounds__(kThreads) k_upload(char* ws, const __grid_constant__ Upload<BYTES> c) {
+  write_chunk(ws, c);
+}
+
 // Plain per-phase kernels, with the same arithmetic as the persistent kernel.
-// Setup: each warp runs one unit (8 per block).  Shading: block b runs unit
-// b, its warp w runs round w of it.
-__global__ void __launch_bounds__(kThreads) k_setup(TableRef tb, int item) {
-  const DItem& it = tb.items[item];
-  const int u = blockIdx.x * kWarps + (threadIdx.x >> 5);
-  if (u < it.units[PH_SETUP]) unit_setup(it, tb.shells + it.shell0, u);
+// Setup: each warp runs one unit (8 per block) on the table it got as a kernel
+// parameter, which block 0 writes to the workspace for the kernels behind: a
+// launch (3 us on the GPU, and the host's share of a small frame) less than
+// with an upload before it.  Shading: block b runs unit b, its warp w runs
+// round w of it.
+__global__ void __launch_bounds__(kThreads) k_setup(char* ws, const __grid_constant__ SmallUpload t,
+                                                    uint32_t shells_off) {
+  if (blockIdx.x == 0) {
+    write_chunk(ws, t);
+    return;
+  }
+  const char* table = reinterpret_cast<const char*>(t.data);
+  const DItem& it = *reinterpret_cast<const DItem*>(table);
+  const int u = (blockIdx.x - 1) * kWarps + (threadIdx.x >> 5);
+  if (u < it.units[PH_SETUP]) unit_setup(it, reinterpret_cast<const DShell*>(table + shells_off) + it.shell0, u);
 }
 
 // Raster: resident blocks only, every warp strides over the item's units (of
@@ -87,13 +102,23 @@ cudaError_t upload(char* ws, const UploadChunk& c, cudaStream_t st) {
   vsd::k_upload<<<1, vsd::kThreads, 0, st>>>(ws, c);
   return cudaGetLastError();
 }
+cudaError_t upload(char* ws, const SmallUpload& c, cudaStream_t st) {
+  vsd::k_upload<<<1, vsd::kThreads, 0, st>>>(ws, c);
+  return cudaGetLastError();
+}
 
-int plain_forward_launches(const int units[4]) { return (units[0] > 0) + (units[1] > 0) + (units[2] > 0); }
-int plain_backward_launches(const int units[4]) { return (units[0] > 0) + (units[2] > 0); }
-
-cudaError_t plain_forward(const TableRef& tb, const int units[4], int tc, bool full, int sms, cudaStream_t st) {
+static void launch_setup(char* ws, const SmallUpload& t, uint32_t shells_off, int units, cudaStream_t st) {
   const int W = vsd::kWarps;
-  if (units[0]) vsd::k_setup<<<(units[0] + W - 1) / W, vsd::kThreads, 0, st>>>(tb, 0);
+  vsd::k_setup<<<1 + (units + W - 1) / W, vsd::kThreads, 0, st>>>(ws, t, shells_off);
+}
+
+int plain_forward_launches(const int units[4]) { return 1 + (units[1] > 0) + (units[2] > 0); }
+int plain_backward_launches(const int units[4]) { return 1 + (units[2] > 0); }
+
+cudaError_t plain_forward(const TableRef& tb, char* ws, const SmallUpload& t, uint32_t shells_off, const int units[4],
+                          int tc, bool full, int sms, cudaStream_t st) {
+  const int W = vsd::kWarps;
+  launch_setup(ws, t, shells_off, units[0], st);
   if (units[1]) {
     const int grid = std::min((units[1] + W - 1) / W, sms * vsd::kRasterBlocks);
     if (full) vsd::k_raster<true><<<grid, vsd::kThreads, vsd::kRasterWarpBytes * W, st>>>(tb, 0);
@@ -104,9 +129,9 @@ cudaError_t plain_forward(const TableRef& tb, const int units[4], int tc, bool f
   return tc_ops(tc).shade(tb, false, full, units[2], vsd::block_smem_bytes(tb.kmax, false, tc), st);
 }
 
-cudaError_t plain_backward(const TableRef& tb, const int units[4], int tc, bool full, cudaStream_t st) {
-  const int W = vsd::kWarps;
-  if (units[0]) vsd::k_setup<<<(units[0] + W - 1) / W, vsd::kThreads, 0, st>>>(tb, 0);
+cudaError_t plain_backward(const TableRef& tb, char* ws, const SmallUpload& t, uint32_t shells_off, const int units[4],
+                           int tc, bool full, cudaStream_t st) {
+  launch_setup(ws, t, shells_off, units[0], st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || !units[2]) return e;
   return tc_ops(tc).shade(tb, true, full, units[2], vsd::block_smem_bytes(tb.kmax, true, tc), st);

@@ -26,15 +26,19 @@ struct TableRef {
 // A slice of the host-built table carried to the device in kernel
 // parameters (so the copy is captured by value in a CUDA graph).
 constexpr int kUploadBytes = 24576;
-struct UploadChunk {
+constexpr int kSmallUploadBytes = 4096;   // the table of a single view, or a short batch's
+template <int BYTES>
+struct Upload {
   uint32_t dst_off;
   uint32_t nbytes;          // multiple of 16
   int32_t reset;            // first chunk: reset next_unit / abort, count launches
   int32_t launches;         // kernels this call enqueues (added to the header)
   int32_t kernel_class;     // first chunk: the call's shading kernels (vs_stats::kernel_class)
   int32_t pad[3];
-  uint4 data[kUploadBytes / 16];
+  uint4 data[BYTES / 16];
 };
+using UploadChunk = Upload<kUploadBytes>;
+using SmallUpload = Upload<kSmallUploadBytes>;
 
 namespace vsk {
 // Launchers of the kernels compiled for one texel class (vsd::TC_*), one
@@ -52,10 +56,15 @@ struct TcOps {
 extern const TcOps kTcAny, kTcRgba, kTcSh0, kTcSh1, kTcSh2, kTcSh3, kTcU80, kTcU81, kTcU82, kTcU83;
 
 cudaError_t upload(char* ws, const UploadChunk& c, cudaStream_t st);
+cudaError_t upload(char* ws, const SmallUpload& c, cudaStream_t st);
+// The launches of a single view; the first one, its setup, carries the table
+// `t` (items at its start, shells at shells_off) and writes it to `ws`.
 int plain_forward_launches(const int units[4]);
 int plain_backward_launches(const int units[4]);
-cudaError_t plain_forward(const TableRef& tb, const int units[4], int tc, bool full, int sms, cudaStream_t st);
-cudaError_t plain_backward(const TableRef& tb, const int units[4], int tc, bool full, cudaStream_t st);
+cudaError_t plain_forward(const TableRef& tb, char* ws, const SmallUpload& t, uint32_t shells_off, const int units[4],
+                          int tc, bool full, int sms, cudaStream_t st);
+cudaError_t plain_backward(const TableRef& tb, char* ws, const SmallUpload& t, uint32_t shells_off, const int units[4],
+                           int tc, bool full, cudaStream_t st);
 cudaError_t persistent(const TableRef& tb, bool bwd, int tc, bool full, int grid, long long spin_limit,
                        cudaStream_t st);
 cudaError_t persistent_occupancy(bool bwd, int tc, bool full, int kmax, int* blocks_per_sm);

@@ -238,7 +238,7 @@ void order_for_locality(std::vector<ItemReq>& req) {
 // and a setup unit.
 struct UnitShape {
   int raster_tris = 32;
-  int shade_rounds = kWarps;
+  int shade_rounds = kShadeWarps;
   int warps = 0;
   int setup_warps = 0;
   bool batch = false;   // a plan of the persistent kernel

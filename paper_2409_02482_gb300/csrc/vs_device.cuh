@@ -19,15 +19,19 @@ namespace vsd {
 // ----------------------------------------------------------------------------
 // tuning constants and table layout
 // ----------------------------------------------------------------------------
-constexpr int kThreads = 256;          // threads per block, all kernels
+constexpr int kThreads = 256;          // threads per block of the setup and raster kernels
 constexpr int kWarps = kThreads / 32;  // a work unit is run by one warp
+// Warps per block of the plain shading kernels.  A block keeps its registers
+// and shared memory until its slowest warp is through, and a view's rounds
+// range from empty to full: with 8 warps 16.4 of 24 were active on average.
+// 800^2 SH2 frame / 1080p baked frame: 182.4 / 378 us with 8 warps, 177.8 /
+// 368.3 with 4, 176.1 / 371.8 with 2, 175.6 / 378.5 with 1.
+constexpr int kShadeWarps = 4;
 constexpr int kSetupVerts = 1024;      // most vertices per setup unit
 constexpr int kClearWords = 16384;     // most visibility words cleared per unit
-constexpr int kShadePixels = 256;      // pixels per shading unit of the plain launches
 // The plain shading launch runs one unit per block, one 32-wide round per
-// warp, so its units are kWarps rounds; the persistent kernel takes any size
-// per item (DItem::shade_rounds).
-static_assert(kShadePixels == 32 * kWarps, "plain units = one round per warp");
+// warp, so its units are kShadeWarps rounds; the persistent kernel takes any
+// size per item (DItem::shade_rounds).
 constexpr int kRasterBlocks = 3;       // resident blocks per SM of the plain raster kernel
 constexpr int kMaxShells = VS_MAX_SHELLS;
 constexpr int kTriBits = 27;           // triangle index bits in a packed fragment
@@ -79,7 +83,7 @@ __host__ __device__ constexpr size_t warp_slice_bytes(int K, bool bwd, int tc) {
   return shade_warp_bytes(K, bwd, tc) > kRasterWarpBytes ? shade_warp_bytes(K, bwd, tc) : kRasterWarpBytes;
 }
 __host__ __device__ constexpr size_t block_smem_bytes(int K, bool bwd, int tc) {
-  return warp_slice_bytes(K, bwd, tc) * kWarps;
+  return warp_slice_bytes(K, bwd, tc) * kShadeWarps;
 }
 
 // Block shape of the persistent kernel, per direction.  Its warps take units

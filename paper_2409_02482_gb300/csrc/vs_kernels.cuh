@@ -28,11 +28,11 @@
 #include "vs_device.cuh"
 #include "vs_kernels.h"
 
-#ifndef VS_BWD_BLOCKS
-#define VS_BWD_BLOCKS 3   // resident 256-thread blocks per SM for kernels with the adjoint
+#ifndef VS_BWD_WARPS
+#define VS_BWD_WARPS 24   // resident warps per SM of the plain shading kernel with the adjoint
 #endif
-#ifndef VS_FWD_BLOCKS
-#define VS_FWD_BLOCKS 3   // ... and for forward-only kernels
+#ifndef VS_FWD_WARPS
+#define VS_FWD_WARPS 24   // ... and of the forward-only one
 #endif
 #ifndef VS_PERS_BWD_BLOCKS
 #define VS_PERS_BWD_BLOCKS 4   // resident blocks per SM of the persistent kernel with the adjoint (pers_threads(true) each)
@@ -1021,7 +1021,7 @@ __device__ __forceinline__ char* warp_smem(int K, bool bwd, int tc) {
 }
 
 template <bool BWD, bool FROM_HITS, int TC, bool FULL>
-__global__ void __launch_bounds__(kThreads, BWD ? VS_BWD_BLOCKS : VS_FWD_BLOCKS) k_shade(TableRef tb, int item) {
+__global__ void __launch_bounds__(32 * kShadeWarps, (BWD ? VS_BWD_WARPS : VS_FWD_WARPS) / kShadeWarps) k_shade(TableRef tb, int item) {
   __shared__ unsigned s_frags;
   const DItem& it = tb.items[item];
   const int w = threadIdx.x >> 5;
@@ -1040,7 +1040,7 @@ __global__ void __launch_bounds__(kThreads, BWD ? VS_BWD_BLOCKS : VS_FWD_BLOCKS)
     const unsigned n = __reduce_add_sync(0xffffffffu, nfrag);
     if ((threadIdx.x & 31) == 0) {
       const unsigned s = atomicAdd(&s_frags, kDone + n) + kDone + n;
-      if (s / kDone == kWarps && s % kDone) atomicAdd(&tb.hdr->frags, (unsigned long long)(s % kDone));
+      if (s / kDone == kShadeWarps && s % kDone) atomicAdd(&tb.hdr->frags, (unsigned long long)(s % kDone));
     }
   } else if (!FROM_HITS) {
     warp_count(&tb.hdr->frags, nfrag);

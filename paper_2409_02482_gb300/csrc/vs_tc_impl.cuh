@@ -37,7 +37,7 @@ cudaError_t tc_persistent(const TableRef& tb, bool bwd, bool full, int grid, lon
 // standalone adjoint from the caller's hit buffer.
 template <bool BWD, bool FULL>
 cudaError_t launch_shade(const TableRef& tb, int blocks, size_t smem, cudaStream_t st) {
-  vsd::k_shade<BWD, BWD, VS_TC, FULL><<<blocks, vsd::kThreads, smem, st>>>(tb, 0);
+  vsd::k_shade<BWD, BWD, VS_TC, FULL><<<blocks, 32 * vsd::kShadeWarps, smem, st>>>(tb, 0);
   return cudaGetLastError();
 }
 

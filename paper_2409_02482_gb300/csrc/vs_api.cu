@@ -613,13 +613,14 @@ vs_tuning lookup_tuning(vs_ctx* ctx, int bwd, int kmax) {
   return ctx->tune_set[bwd][kmax] ? ctx->tune[bwd][kmax] : default_tuning();
 }
 
-// Warps resident in the plain raster kernel, and in the persistent kernels
-// to within a sixth.
-int resident_warps(const vs_ctx* ctx) { return ctx->num_sms * kRasterBlocks * kWarps; }
+// Warps resident in the plain raster kernel, and (to within a sixth) in the
+// persistent ones.
+int plain_warps(const vs_ctx* ctx) { return ctx->num_sms * kRasterBlocks * kWarps; }
+int batch_warps(const vs_ctx* ctx) { return ctx->num_sms * 24; }
 
 UnitShape plain_shape(const vs_ctx* ctx) {
   UnitShape u;
-  u.warps = u.setup_warps = resident_warps(ctx);
+  u.warps = u.setup_warps = plain_warps(ctx);
   return u;
 }
 
@@ -628,7 +629,7 @@ UnitShape shape_of(const vs_ctx* ctx, const vs_tuning& t) {
   u.raster_tris = t.raster_tris;
   u.shade_rounds = t.shade_pixels / 32;
   u.batch = true;
-  u.warps = resident_warps(ctx);
+  u.warps = batch_warps(ctx);
   return u;
 }
 

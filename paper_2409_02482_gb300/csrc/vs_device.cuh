@@ -32,7 +32,9 @@ constexpr int kClearWords = 16384;     // most visibility words cleared per unit
 // The plain shading launch runs one unit per block, one 32-wide round per
 // warp, so its units are kShadeWarps rounds; the persistent kernel takes any
 // size per item (DItem::shade_rounds).
-constexpr int kRasterBlocks = 3;       // resident blocks per SM of the plain raster kernel
+// Resident blocks per SM of the plain raster kernel: 64 registers (800^2 frame
+// of 7 x 200 k triangles: 177.5 us with 3, 172 with 4, 174 with 5).
+constexpr int kRasterBlocks = 4;
 constexpr int kMaxShells = VS_MAX_SHELLS;
 constexpr int kTriBits = 27;           // triangle index bits in a packed fragment
 constexpr int kMaxTris = 1 << kTriBits;
@@ -78,7 +80,7 @@ __host__ __device__ constexpr size_t shade_warp_bytes(int K, bool bwd, int tc) {
           128 * (size_t)pixel_basis(tc, bwd) + 15) &
          ~(size_t)15;
 }
-constexpr size_t kRasterWarpBytes = 32 * (64 + 8 + 4);   // TriS, TriPos, start per triangle
+constexpr size_t kRasterWarpBytes = 32 * 81;   // one TriS and owner per triangle of a round
 __host__ __device__ constexpr size_t warp_slice_bytes(int K, bool bwd, int tc) {
   return shade_warp_bytes(K, bwd, tc) > kRasterWarpBytes ? shade_warp_bytes(K, bwd, tc) : kRasterWarpBytes;
 }

@@ -118,32 +118,47 @@ static __device__ __forceinline__ void raster_clipped(const DShell& s, const DCa
 // pixel (xlo + dx, ylo + dy).  The bound is on the triangle's extent and not
 // on the pixels of its box: a 14 x 14 pixel triangle of a coarse mesh walks
 // with the others of its round (it used to be walked alone, in 64 bits).
+// e_0 + e_1 + e_2 is the same at every point, S, so two edges are kept; the
+// depth's numerator sum e_j q_j is linear in the pixel as well and kept as
+// its three 64-bit coefficients.  A lane takes its record by five 16-byte
+// loads, free of bank conflicts at 80 bytes apart.  A lane writes the record
+// to its own slot as soon as it has set the triangle up, and the pairs find it
+// through a list of owners: kept in registers until the prefix sum said where
+// it goes, it made ptxas spill 130 to 290 bytes in the persistent kernels.
+// With the integer divisions by the box width and the conversions of e_j and
+// q_j (at a quarter of the FP32 rate) gone as well: 800^2 frame 177.6 ->
+// 167.3 us, 32 views forward 4.47 -> 4.40 ms, fused step over 8 uneven assets
+// 4.54 -> 4.34 ms, fitting step of 24 views 8.37 -> 8.44 ms.
 constexpr int kNarrow = 64 * 256;
-struct TriS {
-  int c[3], gx[3], gy[3];
-  unsigned q[3];
+struct alignas(16) TriS {
+  int c0, c1, gx0, gx1;
+  int gy0, gy1, S;
+  float rS;            // 1 / S
+  long long N0, Nx, Ny;
   int tl_bw;           // bits 0-2: top-left edges; bits 8+: box width
-  float rbw;           // 1 / box width
-  float rS;            // 1 / S, S = sum of the edge values = twice the area
-  int t;
+  unsigned mbw;        // see box_row
+  int t, xlo, ylo;     // triangle, box origin
+  int start;           // first pair of the triangle in its round
 };
-struct TriPos {        // box origin of a record
-  int xlo, ylo;
-};
+static_assert((sizeof(TriS) + 1) * 32 == kRasterWarpBytes, "record size");
 
-// floor(sum_j e_j q_j / S) for the 32-bit edge values of a narrow triangle;
-// same estimate-and-correct scheme as depth_key_r.  The estimate is within
-// ~640 of the quotient, so |R| < 2^10 S: from S = 2^21 on R is taken to FP32
-// in units of 2^10 (a thousandth of S), below it fits 32 bits.  (A 64-bit
-// integer converted to FP32 runs on the FP64 pipe, a 64th of the FP32 rate.)
-__device__ __forceinline__ unsigned depth_key32(const unsigned q[3], const int e[3], int S, float rS) {
-  const unsigned long long N = (unsigned long long)(unsigned)e[0] * q[0] +
-                               (unsigned long long)(unsigned)e[1] * q[1] +
-                               (unsigned long long)(unsigned)e[2] * q[2];
-  const float est = fmaf((float)e[0], (float)q[0], fmaf((float)e[1], (float)q[1], (float)e[2] * (float)q[2])) * rS;
-  const unsigned qmin = min(q[0], min(q[1], q[2])), qmax = max(q[0], max(q[1], q[2]));
-  unsigned Q = (unsigned)fminf(fmaxf(est, (float)qmin), (float)qmax);
-  Q = min(max(Q, qmin), qmax);
+// Row of pixel `local` in a box of width bw <= 64 (at most 64 rows):
+// floor(local / bw) = local m >> 20 with m = floor(2^20 / bw) + 1 (or + 2,
+// where the division rounds up), because 0 < m bw - 2^20 <= 128 and
+// local < 2^12.
+__device__ __forceinline__ unsigned box_rows(int bw) { return (unsigned)(1048576.0f / (float)bw) + 1u; }
+__device__ __forceinline__ int box_row(int local, unsigned m) { return (int)(((unsigned)local * m) >> 20); }
+
+// floor(N / S) for the numerator N = sum_j e_j q_j < 2^62 and the edge sum
+// S < 2^30 of a narrow triangle, rS ~ 1 / S; same estimate-and-correct scheme
+// as depth_key_r.  The estimate N rS has a relative error below 2^-21, so it
+// is within 2^10 of the quotient (below 2^31) and |R| < 2^10 S: from S = 2^21
+// on R is taken to FP32 in units of 2^10 (a thousandth of S), below it fits
+// 32 bits.  (A 64-bit integer converted to FP32 runs on the FP64 pipe, a 64th
+// of the FP32 rate, and a 32-bit one at a quarter of it: N takes two
+// conversions where e_j and q_j took six.)
+__device__ __forceinline__ unsigned depth_key32(unsigned long long N, int S, float rS) {
+  unsigned Q = (unsigned)(u64_to_float(N) * rS);
   long long R = (long long)(N - (unsigned long long)Q * (unsigned)S);
   const bool big = S >= (1 << 21);
   const int dQ = (int)floorf((float)(int)(R >> (big ? 10 : 0)) * (big ? 1024.0f * rS : rS));
@@ -154,6 +169,28 @@ __device__ __forceinline__ unsigned depth_key32(const unsigned q[3], const int e
 #pragma unroll 1
   for (int i = 0; i < 4 && R >= S; ++i) { ++Q; R -= S; }
   return Q;
+}
+
+// The record of narrow triangle t but for its start.
+__device__ __forceinline__ void write_record(const Tri& T, int t, TriS* r) {
+  // e_j at the box's first pixel centre, and S = twice the area = e_0 at vertex 0
+  const int ox = 256 * T.xlo + 128, oy = 256 * T.ylo + 128, bw = T.xhi - T.xlo + 1;
+  const int ex0 = T.X[1] - T.X[2], ey0 = T.Y[1] - T.Y[2];   // edge 0: vertex 2 -> 1
+  const int ex1 = T.X[2] - T.X[0], ey1 = T.Y[2] - T.Y[0];   // edge 1: vertex 0 -> 2
+  const int c0 = ex0 * (oy - T.Y[2]) - ey0 * (ox - T.X[2]), c1 = ex1 * (oy - T.Y[0]) - ey1 * (ox - T.X[0]);
+  const int gx0 = -ey0 * 256, gx1 = -ey1 * 256, gy0 = ex0 * 256, gy1 = ex1 * 256;
+  const int S = ex0 * (T.Y[0] - T.Y[2]) - ey0 * (T.X[0] - T.X[2]);
+  const int q02 = (int)(T.q[0] - T.q[2]), q12 = (int)(T.q[1] - T.q[2]);
+  int4* d = reinterpret_cast<int4*>(r);
+  d[0] = make_int4(c0, c1, gx0, gx1);
+  d[1] = make_int4(gy0, gy1, S, __float_as_int(1.0f / (float)S));
+  const long long N0 = (long long)c0 * q02 + (long long)c1 * q12 + (long long)S * (int)T.q[2];
+  const long long Nx = (long long)gx0 * q02 + (long long)gx1 * q12, Ny = (long long)gy0 * q02 + (long long)gy1 * q12;
+  d[2] = make_int4((int)N0, (int)(N0 >> 32), (int)Nx, (int)(Nx >> 32));
+  d[3] = make_int4((int)Ny, (int)(Ny >> 32), T.tl[0] | (T.tl[1] << 1) | (T.tl[2] << 2) | (bw << 8), (int)box_rows(bw));
+  r->t = t;
+  r->xlo = T.xlo;
+  r->ylo = T.ylo;
 }
 
 // Per-lane triangle counts of a raster unit (or of a warp of the plain
@@ -180,57 +217,35 @@ template <bool FULL>
 __device__ __forceinline__ void raster_round(const DItem& it, const DShell& s, int t0, int tend, const int3 ix, int part,
                                              int lg, unsigned long long* vis, char* smem, RasterCounts& rc) {
   TriS* s_tri = reinterpret_cast<TriS*>(smem);
-  TriPos* s_pos = reinterpret_cast<TriPos*>(smem + sizeof(TriS) * 32);
-  int* s_start = reinterpret_cast<int*>(smem + (sizeof(TriS) + sizeof(TriPos)) * 32);
+  unsigned char* s_own = reinterpret_cast<unsigned char*>(smem + 32 * sizeof(TriS));   // triangles with pixels, in order
   const unsigned kAll = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int t = t0 + lane;
   const int W = it.cam.W;
-  unsigned front = 0, back = 0, nearc = 0, guard = 0, large = 0, bad = 0, clip = 0, wide = 0;
+  const unsigned one = part == 0;   // warps that share a round count it once
+  bool wide = false, clip = false;
   int npx = 0;
-  TriS r;
-  TriPos pos;
+  Tri T;
   if (t < tend) {
-    Tri T;
     const int why = load_tri(s, it.cam, ix, T);
     if (why == 0) {
-      front = 1;
+      rc.fb += one;
       const int bw = T.xhi - T.xlo + 1, bh = T.yhi - T.ylo + 1;
       if (bw > 0 && bh > 0) {
-        large = bw * bh > kLargePixels;
+        if (bw * bh > kLargePixels) rc.lc += one;
         const int ext = max(max(max(T.X[0], T.X[1]), T.X[2]) - min(min(T.X[0], T.X[1]), T.X[2]),
                             max(max(T.Y[0], T.Y[1]), T.Y[2]) - min(min(T.Y[0], T.Y[1]), T.Y[2]));
-        if (ext < kNarrow) {
+        wide = ext >= kNarrow;
+        if (!wide) {
           npx = bw * bh;
-          const int ox = 256 * T.xlo + 128, oy = 256 * T.ylo + 128;
-          int S = 0;
-#pragma unroll
-          for (int j = 0; j < 3; ++j) {
-            const int a = (j + 2) % 3, b = (j + 1) % 3;
-            const int ax = T.X[a] - ox, ay = T.Y[a] - oy;
-            const int ex = T.X[b] - T.X[a], ey = T.Y[b] - T.Y[a];
-            r.c[j] = ex * (0 - ay) - ey * (0 - ax);
-            r.gx[j] = -ey * 256;
-            r.gy[j] = ex * 256;
-            r.q[j] = T.q[j];
-            S += r.c[j];
-          }
-          // S = e_0 + e_1 + e_2 is the same at every point
-          r.tl_bw = T.tl[0] | (T.tl[1] << 1) | (T.tl[2] << 2) | (bw << 8);
-          r.rbw = 1.0f / (float)bw;
-          r.rS = 1.0f / (float)S;
-          r.t = t;
-          pos.xlo = T.xlo;
-          pos.ylo = T.ylo;
-        } else {
-          wide = 1;
+          write_record(T, t, s_tri + lane);
         }
       }
-    } else if (why == 1) back = 1;
-    else if (why == 2) nearc = 1;
-    else if (why == 3) guard = 1;
-    else if (why == 5) clip = 1;
-    else bad = 1;
+    } else if (why == 1) rc.fb += one << 16;
+    else if (why == 2) rc.ng += one;
+    else if (why == 3) rc.ng += one << 16;
+    else if (why == 5) { rc.lc += one << 16; clip = true; }
+    else rc.bad = 1;
   }
   // compact the non-empty boxes and take the exclusive prefix of their sizes
   const unsigned ne = __ballot_sync(kAll, npx > 0);
@@ -244,10 +259,8 @@ __device__ __forceinline__ void raster_round(const DItem& it, const DShell& s, i
     const int total = __shfl_sync(kAll, pre, 31);
     const int start = pre - npx;
     if (npx > 0) {
-      const int cpos = __popc(ne & ((1u << lane) - 1u));
-      s_tri[cpos] = r;
-      s_pos[cpos] = pos;
-      s_start[cpos] = start;
+      s_tri[lane].start = start;
+      s_own[__popc(ne & ((1u << lane) - 1u))] = (unsigned char)lane;
     }
     __syncwarp();
     const unsigned le = (lane == 31) ? kAll : ((2u << lane) - 1u);
@@ -257,37 +270,27 @@ __device__ __forceinline__ void raster_round(const DItem& it, const DShell& s, i
       const unsigned bits = __reduce_or_sync(kAll, b);
       const int slot = w0 + lane;
       if (slot < total) {
-        const int o = lg ? 0 : carry + __popc(bits & le) - 1;
+        const int o = s_own[lg ? 0 : carry + __popc(bits & le) - 1];
         const TriS& q = s_tri[o];
-        const int local = slot - s_start[o];
-        const int bwq = q.tl_bw >> 8;
-        const int dy = (int)(((float)local + 0.5f) * q.rbw);
-        const int dx = local - dy * bwq;
-        int e[3];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) e[j] = q.c[j] + q.gx[j] * dx + q.gy[j] * dy;
-        if ((e[0] + (q.tl_bw & 1) > 0) && (e[1] + ((q.tl_bw >> 1) & 1) > 0) && (e[2] + ((q.tl_bw >> 2) & 1) > 0)) {
-          const TriPos p = s_pos[o];
-          const int S = e[0] + e[1] + e[2];
-          red_max_vis(vis + (size_t)(p.ylo + dy) * W + (p.xlo + dx), vis_key(depth_key32(q.q, e, S, q.rS), q.t));
+        const int local = slot - q.start;
+        const int dy = box_row(local, q.mbw);
+        const int dx = local - dy * (q.tl_bw >> 8);
+        const int e0 = q.c0 + q.gx0 * dx + q.gy0 * dy, e1 = q.c1 + q.gx1 * dx + q.gy1 * dy;
+        const int e2 = q.S - e0 - e1;
+        if ((e0 + (q.tl_bw & 1) > 0) && (e1 + ((q.tl_bw >> 1) & 1) > 0) && (e2 + ((q.tl_bw >> 2) & 1) > 0)) {
+          const unsigned long long N = (unsigned long long)(q.N0 + q.Nx * dx + q.Ny * dy);
+          red_max_vis(vis + (size_t)(q.ylo + dy) * W + (q.xlo + dx), vis_key(depth_key32(N, q.S, q.rS), q.t));
         }
       }
       carry += __popc(bits);
     }
   }
-  if (part == 0) {
-    rc.fb += front | (back << 16);
-    rc.ng += nearc | (guard << 16);
-    rc.lc += large | (clip << 16);
-  }
-  rc.bad |= bad;
   // wide triangles: the warp strides over each one's screen box
   unsigned lm = __ballot_sync(kAll, wide);
   while (lm) {
     const int l = __ffs(lm) - 1;
     lm &= lm - 1;
     const int3 iq = make_int3(__shfl_sync(kAll, ix.x, l), __shfl_sync(kAll, ix.y, l), __shfl_sync(kAll, ix.z, l));
-    Tri T;
     if (load_tri(s, it.cam, iq, T) != 0) continue;
     const int bw = T.xhi - T.xlo + 1, bh = T.yhi - T.ylo + 1;
     const int npq = bw * bh;

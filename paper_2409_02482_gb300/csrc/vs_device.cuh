@@ -57,9 +57,9 @@ __host__ __device__ constexpr int pixel_basis(int tc, bool bwd) {
 }
 
 // Dynamic shared memory of a shading warp for up to K shells: a fragment
-// list of frag_cap(K, bwd) entries -- [frag float4][entry u32][alpha_w
-// float][lane|shell u16] and, for the adjoint only, [fractions float2][T
-// float] -- and, when the list is shorter than a round's worst case (32 K),
+// list of frag_cap(K, bwd) entries -- [frag float4][lane|shell u16], for the
+// adjoint [frag float4][entry u32][alpha_w float][lane|shell u16][fractions
+// float2][T float] -- and, when the list is shorter than a round's worst case (32 K),
 // the round's hit table (32 K ints) in front of it, and behind it, for the
 // adjoint, the SH basis of the round's 32 pixels (pixel_basis values each;
 // carved in shade_round).
@@ -76,7 +76,7 @@ __host__ __device__ constexpr int frag_cap(int K, bool bwd) {
   return (bwd && kFragCap < 32 * K) ? kFragCap : 32 * K;
 }
 __host__ __device__ constexpr size_t shade_warp_bytes(int K, bool bwd, int tc) {
-  return ((frag_cap(K, bwd) < 32 * K ? 128 * (size_t)K : 0) + (bwd ? 38 : 26) * (size_t)frag_cap(K, bwd) +
+  return ((frag_cap(K, bwd) < 32 * K ? 128 * (size_t)K : 0) + (bwd ? 38 : 18) * (size_t)frag_cap(K, bwd) +
           128 * (size_t)pixel_basis(tc, bwd) + 15) &
          ~(size_t)15;
 }
@@ -94,13 +94,14 @@ __host__ __device__ constexpr size_t block_smem_bytes(int K, bool bwd, int tc) {
 // The fused forward + adjoint runs 5-warp blocks, 4 per SM: 20 warps at 96
 // registers (measured 0.7 % faster on the C2 fitting step than 24 warps at
 // 80 registers, which spill ~2x more; 16 warps at 128 registers, no spill,
-// 4 % slower).  The forward keeps 8-warp blocks, 3 per SM (24 warps at 80
-// registers: 7 % faster than 20 warps at 96).
+// 4 % slower).  The forward runs 7-warp blocks, 4 per SM: 28 warps at 72
+// registers (32 views at 800^2 4.30 ms, 4 in 4K 10.36 ms; 24 warps at 80
+// registers 4.43 / 10.45 ms, 32 at 64 4.47 / 10.58, 21 at 96 4.62 / 10.34).
 #ifndef VS_PERS_BWD_WARPS
 #define VS_PERS_BWD_WARPS 5
 #endif
 #ifndef VS_PERS_FWD_WARPS
-#define VS_PERS_FWD_WARPS 8
+#define VS_PERS_FWD_WARPS 7
 #endif
 __host__ __device__ constexpr int pers_warps(bool bwd) { return bwd ? VS_PERS_BWD_WARPS : VS_PERS_FWD_WARPS; }
 __host__ __device__ constexpr int pers_threads(bool bwd) { return 32 * pers_warps(bwd); }

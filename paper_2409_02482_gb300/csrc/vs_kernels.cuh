@@ -1007,10 +1007,11 @@ __device__ __forceinline__ void shade_round(const DItem& it, const DShell* sh, i
 
 // Shading unit: 32 * it.shade_rounds consecutive pixels in rounds of 32;
 // this warp runs rounds [r0, r1).  `wb` is the warp's shared-memory slice.
-// Returns the lane's shaded fragments.
+// Returns the lane's shaded fragments; the unit's loss is added to *loss_sum
+// by lane 0.
 template <bool BWD, bool FROM_HITS, int TC, bool FULL>
 __device__ __forceinline__ unsigned unit_shade(const DItem& it, const DShell* sh, int u, WsHeader* hdr, char* wb, int K,
-                                               int r0, int r1) {
+                                               int r0, int r1, float* loss_sum) {
   const unsigned kAll = 0xffffffffu;
   const int HW = it.cam.W * it.cam.H;
   unsigned nfrag = 0, bad = 0;
@@ -1026,7 +1027,7 @@ __device__ __forceinline__ unsigned unit_shade(const DItem& it, const DShell* sh
     if (it.loss && (it.flags & (VS_FLAG_LOSS_L2 | VS_FLAG_LOSS_L1))) {
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(kAll, loss, o);
-      if (lane == 0 && loss != 0.0f) atomicAdd(it.loss, loss);
+      if (lane == 0) *loss_sum += loss;
     }
   }
   return nfrag;
@@ -1052,8 +1053,10 @@ __global__ void __launch_bounds__(32 * kShadeWarps, (BWD ? VS_BWD_WARPS : VS_FWD
     if (threadIdx.x == 0) s_frags = 0;
     __syncthreads();
   }
+  float loss = 0.0f;
   const unsigned nfrag = unit_shade<BWD, FROM_HITS, TC, FULL>(it, tb.shells + it.shell0, blockIdx.x, tb.hdr,
-                                                              warp_smem(tb.kmax, BWD, TC), tb.kmax, w, w + 1);
+                                                              warp_smem(tb.kmax, BWD, TC), tb.kmax, w, w + 1, &loss);
+  if (BWD && loss != 0.0f) atomicAdd(it.loss, loss);
   if (kBlockCount) {   // one addition to the header per block, by its last warp
     constexpr unsigned kDone = 1u << 24;   // warps that are through; below, their fragments
     const unsigned n = __reduce_add_sync(0xffffffffu, nfrag);
@@ -1124,6 +1127,19 @@ __global__ void __launch_bounds__(pers_threads(BWD), BWD ? VS_PERS_BWD_BLOCKS : 
   __shared__ unsigned s_count[pers_warps(BWD)][8];
   unsigned* const my_count = &s_count[threadIdx.x >> 5][lane & 7];
   if (lane < 8) *my_count = 0;
+  // the warp's part of the loss of the item that it last shaded, added to the
+  // item's when the next one comes: the units of the last item are small and
+  // many, and an FP32 sum of them one by one would be the less exact
+  __shared__ float s_loss[pers_warps(BWD)];
+  float* const my_loss = &s_loss[threadIdx.x >> 5];
+  int loss_item = -1;
+  if (lane == 0) *my_loss = 0.0f;
+  auto flush_loss = [&]() {
+    if (lane == 0 && *my_loss != 0.0f) {
+      atomicAdd(tb.items[loss_item].loss, *my_loss);
+      *my_loss = 0.0f;
+    }
+  };
   // the item whose phase (setup, raster) a warp of this block last saw done,
   // by item modulo 4
   __shared__ int s_seen[NPH - 1][4];
@@ -1189,7 +1205,11 @@ __global__ void __launch_bounds__(pers_threads(BWD), BWD ? VS_PERS_BWD_BLOCKS : 
         break;
       }
       default: {
-        const unsigned n = unit_shade<BWD, false, TC, FULL>(it, sh, u, hdr, smem, tb.kmax, 0, it.shade_rounds);
+        if (BWD && loss_item != j) {
+          flush_loss();
+          loss_item = j;
+        }
+        const unsigned n = unit_shade<BWD, false, TC, FULL>(it, sh, u, hdr, smem, tb.kmax, 0, it.shade_rounds, my_loss);
         const unsigned frags = __reduce_add_sync(kAll, n);
         count(lane == 6 ? frags : 0);
       }
@@ -1197,6 +1217,7 @@ __global__ void __launch_bounds__(pers_threads(BWD), BWD ? VS_PERS_BWD_BLOCKS : 
     __syncwarp();
     if (lane == 0) red_release_add(tb.done + j * NPH + ph, 1);   // after the whole warp's writes
   }
+  if (BWD) flush_loss();
   if (lane < kCounters && *my_count) atomicAdd(counter(hdr, lane), (unsigned long long)*my_count);
 }
 

@@ -402,7 +402,6 @@ vs_status make_plan(const ItemReq* req, int n, const float* bg, int do_bwd, bool
       if (j == n - 1)
         while (it.shade_rounds > 1 && (long long)HW < 32ll * it.shade_rounds * shape.warps) it.shade_rounds /= 2;
     }
-    const int shade_per_unit = 32 * it.shade_rounds;
     setup_shape(verts, (long long)(o.k * HW), here, &it.setup_verts, &it.clear_words);
     it.setup_pre[0] = 0;
     it.raster_pre[0] = 0;
@@ -449,7 +448,9 @@ vs_status make_plan(const ItemReq* req, int n, const float* bg, int do_bwd, bool
     it.clear_units = clear_vis ? (int)((vis_words + it.clear_words - 1) / it.clear_words) : 0;
     it.units[PH_SETUP] = it.clear_units + it.setup_pre[o.k];
     it.units[PH_RASTER] = clear_vis ? it.raster_pre[o.k] << it.raster_lg : 0;
-    it.units[PH_SHADE] = (int)((HW + shade_per_unit - 1) / shade_per_unit);
+    const int tw = shape.batch ? kBatchTile : kPlainTile, th = 32 / tw;   // of a shading round
+    const long long rounds = (long long)((c.width + tw - 1) / tw) * ((c.height + th - 1) / th);
+    it.units[PH_SHADE] = (int)((rounds + it.shade_rounds - 1) / it.shade_rounds);
     sidx += o.k;
   }
   P.total = align256(off);

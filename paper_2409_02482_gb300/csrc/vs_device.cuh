@@ -35,6 +35,14 @@ constexpr int kClearWords = 16384;     // most visibility words cleared per unit
 // Resident blocks per SM of the plain raster kernel: 64 registers (800^2 frame
 // of 7 x 200 k triangles: 177.5 us with 3, 172 with 4, 174 with 5).
 constexpr int kRasterBlocks = 4;
+// Width of a shading round's tile of 32 pixels.  A compact tile's footprints
+// share more texels and triangles, a row's accesses to visibility words, hits
+// and image are longer.  Widths 32 / 16 / 8 / 4: 800^2 SH2 frame 164.8 / 163.3
+// / 161.2 / 164.1 us, 1080p baked frame 349 / 346 / 342 / 345; in the batch,
+// where views overlap, 32 views at 800^2 4.29 / 4.30 / 4.33 / 4.56 ms, fitting
+// step of 24 views 8.28 / 8.31 / 8.31 / 8.48, 4 views in 4K 10.09 / 10.50 /
+// 10.88 / 11.7.
+constexpr int kPlainTile = 8, kBatchTile = 32;
 constexpr int kMaxShells = VS_MAX_SHELLS;
 constexpr int kTriBits = 27;           // triangle index bits in a packed fragment
 constexpr int kMaxTris = 1 << kTriBits;

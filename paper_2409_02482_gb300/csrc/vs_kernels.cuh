@@ -553,10 +553,17 @@ __device__ __forceinline__ Footprint unpack_footprint(unsigned xy, float2 fr) {
   return f;
 }
 
+// Pixel of lane l in a shading round's tile of TW x 32 / TW pixels at `tile`.
+template <int TW>
+__device__ __forceinline__ int tile_x(int2 tile, unsigned l) { return tile.x + (int)(l % TW); }
+template <int TW>
+__device__ __forceinline__ int tile_y(int2 tile, unsigned l) { return tile.y + (int)(l / TW); }
+
 // alpha_w of the fragments [0, total) of a shading round (lane-strided),
 // from the packed (shell, triangle) entries; entry j and its result sit at
 // `stride` words times j.
-static __device__ __noinline__ void atten_pass(const DCam& cam, const DShell* sh, int pbase, const int* sent, int stride,
+template <int TW>
+static __device__ __noinline__ void atten_pass(const DCam& cam, const DShell* sh, int2 tile, const int* sent, int stride,
                                                const unsigned short* spl, float* saw, int total) {
   const int lane = threadIdx.x & 31;
   for (int j = lane; j < total; j += 32) {
@@ -569,8 +576,7 @@ static __device__ __noinline__ void atten_pass(const DCam& cam, const DShell* sh
     const int idx[3] = {__ldg(ip), __ldg(ip + 1), __ldg(ip + 2)};
     if ((unsigned)idx[0] >= (unsigned)s.nv || (unsigned)idx[1] >= (unsigned)s.nv || (unsigned)idx[2] >= (unsigned)s.nv)
       continue;
-    const int pp = pbase + (spl[j] & 31);
-    const int y = pp / cam.W, x = pp - y * cam.W;
+    const int x = tile_x<TW>(tile, spl[j] & 31), y = tile_y<TW>(tile, spl[j] & 31);
     saw[j * stride] = alpha_atten(s.pos, idx, ray_dir(cam, x, y));
   }
 }
@@ -602,8 +608,8 @@ constexpr unsigned kClipFrag = 0x4000u;   // triangle to clip at the near plane 
 // part used at its pixel, footprint, texel fetch; like the fetch loop of
 // shade_round, out of line because it is rare.  The forward finds the entry
 // and alpha_w in the place of the colour.
-template <bool BWD, int TC>
-static __device__ __forceinline__ void shade_clipped(const DItem& it, const DShell* sh, int pbase, int j, const int* sent,
+template <bool BWD, int TC, int TW>
+static __device__ __forceinline__ void shade_clipped(const DItem& it, const DShell* sh, int2 tile, int j, const int* sent,
                                                   unsigned short* spl, float4* sfrag, unsigned* sxy, float2* sfxy,
                                                   unsigned* nfrag, unsigned* bad) {
   const int e = BWD ? sent[j] : __float_as_int(sfrag[j].x);
@@ -611,9 +617,7 @@ static __device__ __forceinline__ void shade_clipped(const DItem& it, const DShe
   const DShell& s = sh[e >> kTriBits];
   const int* ip = s.tris + 3 * (size_t)(e & (kMaxTris - 1));
   const int idx[3] = {__ldg(ip), __ldg(ip + 1), __ldg(ip + 2)};   // checked in range by load_tri_shade
-  const int pp = pbase + (spl[j] & 31);
-  const int W = it.cam.W;
-  const int y = pp / W, x = pp - y * W;
+  const int x = tile_x<TW>(tile, spl[j] & 31), y = tile_y<TW>(tile, spl[j] & 31);
   Tri T;
   float2 uv[3];
   Frag fr = {0.f, 0.f, 0.f, 0.f};
@@ -636,13 +640,13 @@ static __device__ __forceinline__ void shade_clipped(const DItem& it, const DShe
     float3 v = make_float3(0.f, 0.f, 1.f);
     if (is_sh<TC>(s)) v = ray_dir(it.cam, x, y);
     fr = fetch_frag<TC, !BWD>(s, f, ix, fx, iy, fy, v);
-    if (it.layers) layer_geom(it, s, idx, e >> kTriBits, pp, ix, fx, iy, fy);
+    if (it.layers) layer_geom(it, s, idx, e >> kTriBits, y * it.cam.W + x, ix, fx, iy, fy);
     ++*nfrag;
   }
   sfrag[j] = make_float4(fr.r, fr.g, fr.b, BWD ? fr.a : fr.a * aw);
 }
 
-// Shading round: 32 consecutive pixels, one per lane.
+// Shading round: a tile of 32 pixels, one per lane.
 //  1. each lane reads its pixel's k visibility words (independent loads)
 //     into a per-shell hit table.  The round then runs in passes over
 //     consecutive lane ranges whose fragments fit the warp's list (one
@@ -692,8 +696,8 @@ static __device__ __forceinline__ void shade_clipped(const DItem& it, const DShe
 static_assert(kMaxShells <= 16, "shell index takes 4 bits of the lane word");
 static_assert(kFragCap >= kMaxShells, "a pixel's fragments must fit one pass");
 
-template <bool BWD, bool FROM_HITS, int TC, bool FULL>
-__device__ __forceinline__ void shade_round(const DItem& it, const DShell* sh, int pbase, char* wb, int K,
+template <bool BWD, bool FROM_HITS, int TC, bool FULL, int TW>
+__device__ __forceinline__ void shade_round(const DItem& it, const DShell* sh, int2 tile, char* wb, int K,
                                             unsigned& nfrag, unsigned& bad, float& loss_acc) {
   const unsigned kAll = 0xffffffffu;
   const int W = it.cam.W, H = it.cam.H;
@@ -714,12 +718,11 @@ __device__ __forceinline__ void shade_round(const DItem& it, const DShell* sh, i
   float* sT = reinterpret_cast<float*>(lb + 34 * C);       // BWD only
   constexpr int NB = pixel_basis(TC, BWD);
   float* sY = reinterpret_cast<float*>(lb + 38 * C);       // NB > 0 only
-  const int p = pbase + lane;
-  const bool pix_ok = p < HW;
+  const int px = tile_x<TW>(tile, lane), py = tile_y<TW>(tile, lane), p = py * W + px;
+  const bool pix_ok = px < W && py < H;
   if constexpr (NB > 0) {   // SH basis of this lane's pixel, shared by its fragments
     if (pix_ok) {
-      const int y = p / W, x = p - y * W;
-      const float3 v = ray_dir(it.cam, x, y);
+      const float3 v = ray_dir(it.cam, px, py);
       float Yb[16];
       sh_basis(TC - TC_SH0, v.x, v.y, v.z, Yb);
 #pragma unroll
@@ -793,7 +796,7 @@ __device__ __forceinline__ void shade_round(const DItem& it, const DShell* sh, i
     // 2a. transparency attenuation, in a pass of its own so that the fetch
     //     loop below keeps its registers
     if (atten) {
-      atten_pass(it.cam, sh, pbase, sent, EST, spl, saw, nf);
+      atten_pass<TW>(it.cam, sh, tile, sent, EST, spl, saw, nf);
       __syncwarp();
     }
 
@@ -805,12 +808,11 @@ __device__ __forceinline__ void shade_round(const DItem& it, const DShell* sh, i
       if constexpr (!BWD) __syncwarp();   // the step's colours may take its entries' place
       if (j < nf) {
         const int i = e >> kTriBits, t = e & (kMaxTris - 1);
-        const int pp = pbase + (spl[j] & 31);
         const DShell& s = sh[i];
         Frag fr = {0.f, 0.f, 0.f, 0.f};
         Tri Tr;
         int idx[3];
-        const int y = pp / W, x = pp - y * W;
+        const int x = tile_x<TW>(tile, spl[j] & 31), y = tile_y<TW>(tile, spl[j] & 31);
         float2 uv[3];
         const int r = t < s.nt ? load_tri_shade(s, t, Tr, idx, uv) : 4;
         if (FULL && r == 2) {
@@ -842,7 +844,7 @@ __device__ __forceinline__ void shade_round(const DItem& it, const DShell* sh, i
             fr = fetch_frag<TC, !BWD>(s, f, ix, fx, iy, fy, v);
           }
           if constexpr (FULL) {
-            if (it.layers) layer_geom(it, s, idx, i, pp, ix, fx, iy, fy);
+            if (it.layers) layer_geom(it, s, idx, i, y * W + x, ix, fx, iy, fy);
           }
           ++nfrag;
         }
@@ -857,7 +859,7 @@ __device__ __forceinline__ void shade_round(const DItem& it, const DShell* sh, i
     // 2c. fragments of triangles clipped at the near plane (rare; out of line)
     if (FULL && __any_sync(kAll, clip_pending)) {
       for (int j = lane; j < nf; j += 32)
-        if (spl[j] & kClipFrag) shade_clipped<BWD, TC>(it, sh, pbase, j, sent, spl, sfrag, sxy, sfxy, &nfrag, &bad);
+        if (spl[j] & kClipFrag) shade_clipped<BWD, TC, TW>(it, sh, tile, j, sent, spl, sfrag, sxy, sfxy, &nfrag, &bad);
       __syncwarp();
     }
 
@@ -992,9 +994,7 @@ __device__ __forceinline__ void shade_round(const DItem& it, const DShell* sh, i
           const Footprint f = unpack_footprint(sxy[j], sfxy[j]);
           float3 v = make_float3(0.f, 0.f, 1.f);
           if (is_sh<TC>(s)) {
-            const int pp = pbase + (int)(pl & 31);
-            const int y = pp / W, x = pp - y * W;
-            v = ray_dir(it.cam, x, y);
+            v = ray_dir(it.cam, tile_x<TW>(tile, pl & 31), tile_y<TW>(tile, pl & 31));
           }
           scatter_frag<TC>(s, f, v, sfrag[j]);
         }
@@ -1005,21 +1005,24 @@ __device__ __forceinline__ void shade_round(const DItem& it, const DShell* sh, i
   }
 }
 
-// Shading unit: 32 * it.shade_rounds consecutive pixels in rounds of 32;
+// Shading unit: it.shade_rounds consecutive tiles (row by row of tiles);
 // this warp runs rounds [r0, r1).  `wb` is the warp's shared-memory slice.
 // Returns the lane's shaded fragments; the unit's loss is added to *loss_sum
 // by lane 0.
-template <bool BWD, bool FROM_HITS, int TC, bool FULL>
+template <bool BWD, bool FROM_HITS, int TC, bool FULL, int TW>
 __device__ __forceinline__ unsigned unit_shade(const DItem& it, const DShell* sh, int u, WsHeader* hdr, char* wb, int K,
                                                int r0, int r1, float* loss_sum) {
   const unsigned kAll = 0xffffffffu;
-  const int HW = it.cam.W * it.cam.H;
+  constexpr int TH = 32 / TW;
+  const int tiles_x = (it.cam.W + TW - 1) / TW, tiles = tiles_x * ((it.cam.H + TH - 1) / TH);
   unsigned nfrag = 0, bad = 0;
   float loss = 0.0f;
   for (int r = r0; r < r1; ++r) {
-    const int pbase = (u * it.shade_rounds + r) * 32;
-    if (pbase >= HW) break;
-    shade_round<BWD, FROM_HITS, TC, FULL>(it, sh, pbase, wb, K, nfrag, bad, loss);
+    const int t = u * it.shade_rounds + r;
+    if (t >= tiles) break;
+    const int ty = t / tiles_x;
+    shade_round<BWD, FROM_HITS, TC, FULL, TW>(it, sh, make_int2((t - ty * tiles_x) * TW, ty * TH), wb, K, nfrag, bad,
+                                              loss);
   }
   const int lane = threadIdx.x & 31;
   if (__any_sync(kAll, bad) && lane == 0) record_error(hdr, VS_ERR_INVALID_ARG);
@@ -1054,8 +1057,8 @@ __global__ void __launch_bounds__(32 * kShadeWarps, (BWD ? VS_BWD_WARPS : VS_FWD
     __syncthreads();
   }
   float loss = 0.0f;
-  const unsigned nfrag = unit_shade<BWD, FROM_HITS, TC, FULL>(it, tb.shells + it.shell0, blockIdx.x, tb.hdr,
-                                                              warp_smem(tb.kmax, BWD, TC), tb.kmax, w, w + 1, &loss);
+  const unsigned nfrag = unit_shade<BWD, FROM_HITS, TC, FULL, kPlainTile>(it, tb.shells + it.shell0, blockIdx.x, tb.hdr,
+                                                                          warp_smem(tb.kmax, BWD, TC), tb.kmax, w, w + 1, &loss);
   if (BWD && loss != 0.0f) atomicAdd(it.loss, loss);
   if (kBlockCount) {   // one addition to the header per block, by its last warp
     constexpr unsigned kDone = 1u << 24;   // warps that are through; below, their fragments
@@ -1209,7 +1212,7 @@ __global__ void __launch_bounds__(pers_threads(BWD), BWD ? VS_PERS_BWD_BLOCKS : 
           flush_loss();
           loss_item = j;
         }
-        const unsigned n = unit_shade<BWD, false, TC, FULL>(it, sh, u, hdr, smem, tb.kmax, 0, it.shade_rounds, my_loss);
+        const unsigned n = unit_shade<BWD, false, TC, FULL, kBatchTile>(it, sh, u, hdr, smem, tb.kmax, 0, it.shade_rounds, my_loss);
         const unsigned frags = __reduce_add_sync(kAll, n);
         count(lane == 6 ? frags : 0);
       }

@@ -259,12 +259,16 @@ constexpr int kUnitPixels = 2048, kLeastTris = 8;
 // every resident warp gets one, else smaller, down to one triangle, which 2,
 // 4 .. 64 warps then share.  A mesh of few triangles has large ones: at 256^2,
 // 3 x 1224 triangles took 253 us in units of 32 (115 warps busy) and take
-// 7 us one by one.
-void raster_shape(long long tris, const UnitShape& shape, int* unit, int* lg) {
+// 7 us one by one.  The items of a batch (n) run beside one another, so a
+// quarter of the warps each is enough, and full rounds: every unit also costs
+// about 3 ns of the words that all warps share (fitting step of 7 views of 2 x
+// 54 k triangles, 809 x 117: 249 us with all warps, 242 with a quarter).
+void raster_shape(long long tris, const UnitShape& shape, int n, int* unit, int* lg) {
   *unit = shape.raster_tris;
   *lg = 0;
-  while (*unit > 1 && tris / *unit < shape.warps) *unit /= 2;
-  while (*unit == 1 && *lg < 6 && (tris << (*lg + 1)) <= shape.warps) ++*lg;
+  const int least = n > 1 ? 32 : 1, warps = shape.warps / std::min(n, 4);
+  while (*unit > least && tris / *unit < warps) *unit /= 2;
+  while (*unit == 1 && *lg < 6 && (tris << (*lg + 1)) <= warps) ++*lg;
 }
 
 // Setup units of an item of `verts` vertices and `words` visibility words to
@@ -388,19 +392,21 @@ vs_status make_plan(const ItemReq* req, int n, const float* bg, int do_bwd, bool
       verts += o.shells[i].num_verts;
     }
     int raster_tris = 0;
-    raster_shape(tris, shape, &raster_tris, &it.raster_lg);
+    raster_shape(tris, shape, n, &raster_tris, &it.raster_lg);
     it.shade_rounds = shape.shade_rounds;
     it.bg[0] = bg ? bg[0] : 0.f; it.bg[1] = bg ? bg[1] : 0.f; it.bg[2] = bg ? bg[2] : 0.f;
     const size_t HW = (size_t)c.width * c.height;
     UnitShape here = shape;
     // the ends of a batch's pipeline, where no other item fills the GPU: the
-    // first item's setup and the last one's shading are cut so that every
-    // warp finds a unit (32 views at 800^2: 4.51 -> 4.47 ms, fitting step of
-    // 24 views 8.42 -> 8.36 ms; four units per warp: 8.42)
+    // first item's setup and the last one's shading are cut (to two rounds at
+    // least) while some warps find no unit.  32 views at 800^2: 4.30 -> 4.27
+    // ms, fitting step of 24 views 8.42 -> 8.37 ms, 8 views of 4 x 361 k
+    // triangles 868 -> 840 us; shading units of one round cost a small fitting
+    // step 3 % (232 -> 241 us).
     if (shape.batch) {
-      if (j == 0) here.setup_warps = shape.warps;
+      if (j == 0) here.setup_warps = shape.warps / 4;
       if (j == n - 1)
-        while (it.shade_rounds > 1 && (long long)HW < 32ll * it.shade_rounds * shape.warps) it.shade_rounds /= 2;
+        while (it.shade_rounds > 2 && (long long)HW < 32ll * it.shade_rounds * shape.warps) it.shade_rounds /= 2;
     }
     setup_shape(verts, (long long)(o.k * HW), here, &it.setup_verts, &it.clear_words);
     it.setup_pre[0] = 0;

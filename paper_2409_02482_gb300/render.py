@@ -38,7 +38,11 @@ def camera_struct(cam) -> vs_camera:
     """vs_camera from any object with world_to_cam (3x4), fx, fy, cx, cy,
     znear, width, height (e.g. synth.Camera)."""
     c = vs_camera()
-    m = torch.as_tensor(cam.world_to_cam, dtype=torch.float32).reshape(-1).tolist()
+    m = cam.world_to_cam
+    if isinstance(m, torch.Tensor):   # values go to FP32 in the assignment below
+        m = [v for row in m.tolist() for v in row] if m.dim() == 2 else m.reshape(-1).tolist()
+    else:
+        m = torch.as_tensor(m, dtype=torch.float32).reshape(-1).tolist()
     for i in range(12):
         c.world_to_cam[i] = m[i]
     c.fx, c.fy, c.cx, c.cy, c.znear = (float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy),
@@ -211,13 +215,17 @@ def render_backward(ctx: Context, obj: ShellObject, cam, ws: torch.Tensor, hits:
     """vs_render_backward: accumulates into (and returns) FP32 texel grads."""
     if grads is None:
         grads = obj.zero_grads()
+    _backward_into(ctx, obj, cam, ws, hits, grad_rgb.contiguous(), [g.data_ptr() for g in grads], bg, loss, flags,
+                   stream)
+    return grads
+
+
+def _backward_into(ctx: Context, obj: ShellObject, cam, ws, hits, grad_rgb, grad_ptrs, bg, loss, flags, stream):
     c = camera_struct(cam)
     bgv = (ctypes.c_float * 3)(*bg)
-    gptrs = (ctypes.c_void_p * obj.k)(*[g.data_ptr() for g in grads])
+    gptrs = (ctypes.c_void_p * obj.k)(*grad_ptrs)
     check(ctx.lib.vs_render_backward(ctx.handle, obj.handle, ctypes.byref(c), bgv, _ptr(hits),
-                                     _ptr(grad_rgb.contiguous()), gptrs, _ptr(loss), _ptr(ws),
-                                     ws.numel(), flags, _stream(stream)))
-    return grads
+                                     _ptr(grad_rgb), gptrs, _ptr(loss), _ptr(ws), ws.numel(), flags, _stream(stream)))
 
 
 class BatchItems:
@@ -365,14 +373,22 @@ class VSRender(torch.autograd.Function):
 
     forward(ctx_, obj, cam, ws, bg, flags, *textures) -> rgba [H,W,4]; the
     hit buffer is saved and the backward recomputes transmittance from it
-    (vs_render_backward, same flags).  Gradients come back in FP32 and
-    autograd casts them to each texture's dtype.
+    (vs_render_backward, same flags).  Gradients are computed in FP32 and come
+    back in each texture's dtype.  One buffer holds all shells' gradients, so
+    that clearing and casting take a launch each: five shells of 1000 x 720
+    SH1 texels at 1001 x 751 spent more host time on the step (460 us) than
+    the GPU.
     """
+
+    # FP32 values to which each shell's part of the buffer is rounded up: parts
+    # start on 256-byte boundaries (128 once cast to FP16)
+    _ROUND = 64
 
     @staticmethod
     def forward(fctx, vctx: Context, obj: ShellObject, cam, ws: torch.Tensor, bg, flags, *textures):
         out, hits = render(vctx, obj, cam, ws, bg=bg, flags=flags)
         fctx.vctx, fctx.obj, fctx.cam, fctx.ws, fctx.bg, fctx.flags = vctx, obj, cam, ws, bg, flags
+        fctx.dtypes = [t.dtype for t in textures]
         fctx.save_for_backward(hits)
         return out
 
@@ -380,8 +396,18 @@ class VSRender(torch.autograd.Function):
     def backward(fctx, grad_out):
         (hits,) = fctx.saved_tensors
         g = grad_out[..., :3].contiguous().float()
-        grads = render_backward(fctx.vctx, fctx.obj, fctx.cam, fctx.ws, hits, g, bg=fctx.bg,
-                                flags=fctx.flags)
+        shapes = fctx.obj.grad_shapes()
+        starts, total = [], 0
+        for h, w, p in shapes:
+            starts.append(total)
+            total += -(-h * w * p // VSRender._ROUND) * VSRender._ROUND
+        flat = torch.zeros(total, dtype=torch.float32, device=hits.device)
+        base = flat.data_ptr()
+        _backward_into(fctx.vctx, fctx.obj, fctx.cam, fctx.ws, hits, g, [base + 4 * a for a in starts], fctx.bg, None,
+                       fctx.flags, None)
+        if len(set(fctx.dtypes)) == 1:
+            flat = flat.to(fctx.dtypes[0])
+        grads = [flat.as_strided(s, (s[1] * s[2], s[2], 1), a) for s, a in zip(shapes, starts)]
         out = []
         for gr, t in zip(grads, fctx.obj.textures):   # gradient pitch -> texel pitch
             p, gp = t.shape[2], gr.shape[2]

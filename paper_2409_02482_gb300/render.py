@@ -374,10 +374,14 @@ class VSRender(torch.autograd.Function):
     forward(ctx_, obj, cam, ws, bg, flags, *textures) -> rgba [H,W,4]; the
     hit buffer is saved and the backward recomputes transmittance from it
     (vs_render_backward, same flags).  Gradients are computed in FP32 and come
-    back in each texture's dtype.  One buffer holds all shells' gradients, so
-    that clearing and casting take a launch each: five shells of 1000 x 720
-    SH1 texels at 1001 x 751 spent more host time on the step (460 us) than
-    the GPU.
+    back in each texture's dtype.  When every texture requires a gradient, one
+    buffer holds those of all shells, so that clearing and casting take a
+    launch each (arrays per shell: 431 us of host time against 378 for a step
+    with five shells of 1000 x 720 SH1 texels at 1001 x 751, whose GPU time is
+    290).  Its parts are tensors of their own, with version counters of their
+    own, but they share its storage: keeping one keeps all (clone a gradient
+    that outlives the others, or that is saved alone).  Otherwise each shell's
+    gradients are an array of their own.
     """
 
     # FP32 values to which each shell's part of the buffer is rounded up: parts
@@ -396,18 +400,24 @@ class VSRender(torch.autograd.Function):
     def backward(fctx, grad_out):
         (hits,) = fctx.saved_tensors
         g = grad_out[..., :3].contiguous().float()
-        shapes = fctx.obj.grad_shapes()
-        starts, total = [], 0
-        for h, w, p in shapes:
-            starts.append(total)
-            total += -(-h * w * p // VSRender._ROUND) * VSRender._ROUND
-        flat = torch.zeros(total, dtype=torch.float32, device=hits.device)
-        base = flat.data_ptr()
-        _backward_into(fctx.vctx, fctx.obj, fctx.cam, fctx.ws, hits, g, [base + 4 * a for a in starts], fctx.bg, None,
-                       fctx.flags, None)
-        if len(set(fctx.dtypes)) == 1:
-            flat = flat.to(fctx.dtypes[0])
-        grads = [flat.as_strided(s, (s[1] * s[2], s[2], 1), a) for s, a in zip(shapes, starts)]
+        if all(fctx.needs_input_grad[6:]):
+            shapes = fctx.obj.grad_shapes()
+            starts, total = [], 0
+            for h, w, p in shapes:
+                starts.append(total)
+                total += -(-h * w * p // VSRender._ROUND) * VSRender._ROUND
+            flat = torch.zeros(total, dtype=torch.float32, device=hits.device)
+            base = flat.data_ptr()
+            _backward_into(fctx.vctx, fctx.obj, fctx.cam, fctx.ws, hits, g, [base + 4 * a for a in starts], fctx.bg,
+                           None, fctx.flags, None)
+            if len(set(fctx.dtypes)) == 1:
+                flat = flat.to(fctx.dtypes[0])
+            # .data: views of one tensor would share its version counter, and a
+            # change of one shell's gradient in place would count as a change of
+            # every other that autograd has saved
+            grads = [flat.as_strided(s, (s[1] * s[2], s[2], 1), a).data for s, a in zip(shapes, starts)]
+        else:
+            grads = render_backward(fctx.vctx, fctx.obj, fctx.cam, fctx.ws, hits, g, bg=fctx.bg, flags=fctx.flags)
         out = []
         for gr, t in zip(grads, fctx.obj.textures):   # gradient pitch -> texel pitch
             p, gp = t.shape[2], gr.shape[2]

@@ -22,6 +22,7 @@
 #include "vs_device.cuh"
 #include "vs_kernels.h"
 #include "vs_ntex.h"
+#include "vs_units.h"
 
 using namespace vsd;
 
@@ -244,33 +245,6 @@ struct UnitShape {
   bool batch = false;   // a plan of the persistent kernel
 };
 
-// A raster unit of a batch is cut, down to kLeastTris triangles, while its
-// shell's triangles would cover more than kUnitPixels pixels if the shell
-// filled the image: the units of a shell of 10 k triangles are then about as
-// long as those of one with 1 M, and the shading of a view does not wait for
-// its last few coarse units.  Fused step over 8 objects with 10 k to 1 M
-// triangles per shell: 7.32 ms with equal units, 4.72 at 32 triangles at
-// least, 4.56 at 8, the same at 1.  kUnitPixels = 1024 halves the units of a
-// 4K view of 9 x 2 M triangles, 10.34 -> 10.70 ms; 1400 to 4096 are within
-// 0.3 % of each other there and at 800^2.
-constexpr int kUnitPixels = 2048, kLeastTris = 8;
-
-// Raster units of an item of `tris` triangles: units of the asked size while
-// every resident warp gets one, else smaller, down to one triangle, which 2,
-// 4 .. 64 warps then share.  A mesh of few triangles has large ones: at 256^2,
-// 3 x 1224 triangles took 253 us in units of 32 (115 warps busy) and take
-// 7 us one by one.  The items of a batch (n) run beside one another, so a
-// quarter of the warps each is enough, and full rounds: every unit also costs
-// about 3 ns of the words that all warps share (fitting step of 7 views of 2 x
-// 54 k triangles, 809 x 117: 249 us with all warps, 242 with a quarter).
-void raster_shape(long long tris, const UnitShape& shape, int n, int* unit, int* lg) {
-  *unit = shape.raster_tris;
-  *lg = 0;
-  const int least = n > 1 ? 32 : 1, warps = shape.warps / std::min(n, 4);
-  while (*unit > least && tris / *unit < warps) *unit /= 2;
-  while (*unit == 1 && *lg < 6 && (tris << (*lg + 1)) <= warps) ++*lg;
-}
-
 // Setup units of an item of `verts` vertices and `words` visibility words to
 // clear: the largest size at which every warp asked for finds one of each
 // kind, but no fewer than 32 vertices (one per lane) and 512 words (8 stores
@@ -367,6 +341,10 @@ vs_status make_plan(const ItemReq* req, int n, const float* bg, int do_bwd, bool
   P.items.assign(n, DItem{});
   P.shells.assign(S, DShell{});
   P.stage_pre.assign((size_t)n + NPH, 0);
+  long long batch_tris = 0;
+  for (int j = 0; j < n; ++j)
+    for (int i = 0; i < req[j].obj->k; ++i) batch_tris += req[j].obj->shells[i].num_tris;
+  const vsu::RasterUnits units = vsu::raster_units(batch_tris, shape.raster_tris, n, shape.warps);
   int sidx = 0;
   for (int j = 0; j < n; ++j) {
     const vs_object& o = *req[j].obj;
@@ -386,13 +364,9 @@ vs_status make_plan(const ItemReq* req, int n, const float* bg, int do_bwd, bool
     it.flags = (int)flags;
     it.do_bwd = do_bwd;
     it.stall = (flags & VS_FLAG_TEST_STALL) ? 1 : 0;
-    long long tris = 0, verts = 0;
-    for (int i = 0; i < o.k; ++i) {
-      tris += o.shells[i].num_tris;
-      verts += o.shells[i].num_verts;
-    }
-    int raster_tris = 0;
-    raster_shape(tris, shape, n, &raster_tris, &it.raster_lg);
+    long long verts = 0;
+    for (int i = 0; i < o.k; ++i) verts += o.shells[i].num_verts;
+    it.raster_lg = units.lg;
     it.shade_rounds = shape.shade_rounds;
     it.bg[0] = bg ? bg[0] : 0.f; it.bg[1] = bg ? bg[1] : 0.f; it.bg[2] = bg ? bg[2] : 0.f;
     const size_t HW = (size_t)c.width * c.height;
@@ -442,10 +416,9 @@ vs_status make_plan(const ItemReq* req, int n, const float* bg, int do_bwd, bool
       s.vsetup = reinterpret_cast<int4*>(ws ? ws + off : nullptr);
       off = align256(off + sizeof(int4) * (size_t)d.num_verts);
       it.setup_pre[i + 1] = it.setup_pre[i] + (d.num_verts + it.setup_verts - 1) / it.setup_verts;
-      s.raster_tris = raster_tris;
+      s.raster_tris = units.tris;
       if (shape.batch)
-        while (s.raster_tris > kLeastTris && s.raster_tris * (long long)HW > (long long)kUnitPixels * d.num_tris)
-          s.raster_tris /= 2;
+        s.raster_tris = vsu::shell_unit(units.tris, d.num_tris, (long long)HW, batch_tris, n, shape.warps);
       it.raster_pre[i + 1] = it.raster_pre[i] + (d.num_tris + s.raster_tris - 1) / s.raster_tris;
     }
     it.vis = reinterpret_cast<unsigned long long*>(ws ? ws + off : nullptr);

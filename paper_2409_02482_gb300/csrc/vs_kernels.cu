@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(kThreads) k_setup(char* ws, const __grid_const
 
 // Raster: resident blocks only, every warp strides over the item's units (of
 // 32 triangles, or fewer where the mesh is too small to give every warp
-// one: see raster_shape).  What bounds it: latency of the dependent index and
+// one: see vs_units.h).  What bounds it: latency of the dependent index and
 // vertex loads and of the walk.  One block per 256 triangles, each of its
 // warps adding its counts to the workspace header by itself, made 87 k
 // atomics on one cache line of an 800^2 view of 7 x 200 k triangles, and they

@@ -37,15 +37,17 @@ struct Enc {
   int L, F, logT, base;
   float growth;
   int res[16];
+  int pairs;   // two features per level and rows on 8-byte boundaries: one load per row
 };
 
 // Level resolutions N_l = floor(N_min b^l), computed on the host in double.
-Enc make_enc(const vs_ntex_config& c) {
+Enc make_enc(const vs_ntex_config& c, const float* table) {
   Enc e{};
   e.L = c.levels;
   e.F = c.features;
   e.logT = c.log2_table;
   e.base = c.base_res;
+  e.pairs = c.features == 2 && (uintptr_t)table % 8 == 0;
   e.growth = c.growth;
   for (int l = 0; l < c.levels; ++l) e.res[l] = (int)std::floor((double)c.base_res * std::pow((double)c.growth, l));
   return e;
@@ -159,7 +161,7 @@ __global__ void __launch_bounds__(kThreads) k_encode(const __grid_constant__ Enc
   uint32_t row[4];
   float w[4];
   corners4(e, l, tx, ty, W, H, row, w);
-  if (e.F == 2) {   // four 8-byte rows, all in flight; the same sums as below
+  if (e.pairs) {   // four 8-byte rows, all in flight; the same sums as below
     const float2* t2 = reinterpret_cast<const float2*>(table) + lt;
     float2 v[4];
 #pragma unroll
@@ -210,13 +212,13 @@ struct TgPlan {
   int pre[17];      // first block of level l
 };
 
-// dst[0 .. F) += v[0 .. F) with vector reductions where F allows (8- and
-// 16-byte aligned rows).
-template <int F>
+// dst[0 .. F) += v[0 .. F), with vector reductions where F allows and the rows
+// are aligned for them (8 bytes for F = 2, 16 for F a multiple of 4).
+template <int F, bool VEC>
 __device__ __forceinline__ void red_row(float* dst, const float* v) {
-  if constexpr (F == 2) {
+  if constexpr (F == 2 && VEC) {
     asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(dst), "f"(v[0]), "f"(v[1]) : "memory");
-  } else if constexpr (F % 4 == 0) {
+  } else if constexpr (F % 4 == 0 && VEC) {
 #pragma unroll
     for (int f = 0; f < F; f += 4)
       asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + f), "f"(v[f]),
@@ -247,7 +249,7 @@ __device__ __forceinline__ void load_row(const float* src, float* v) {
   }
 }
 
-template <int F>
+template <int F, bool VEC>
 __global__ void __launch_bounds__(kTgThreads) k_table_grad(const __grid_constant__ Enc e,
                                                            const __grid_constant__ TgPlan p, const float* __restrict__ dX,
                                                            long long sl, int si, int W, int H, int n0, int count,
@@ -298,7 +300,7 @@ __global__ void __launch_bounds__(kTgThreads) k_table_grad(const __grid_constant
           if (!any) continue;
           const int vx = cx + dx, vy = cur + dy;
           if (direct) {
-            red_row<F>(tl + (size_t)table_row(e, l, (uint32_t)vx, (uint32_t)vy) * F, v);
+            red_row<F, VEC>(tl + (size_t)table_row(e, l, (uint32_t)vx, (uint32_t)vy) * F, v);
           } else {
             float* q = box + ((vy - by0) * bxn + (vx - bx0)) * F;
 #pragma unroll
@@ -348,7 +350,7 @@ __global__ void __launch_bounds__(kTgThreads) k_table_grad(const __grid_constant
       }
       if (!any) continue;
       const int vy = by0 + i / bxn, vx = bx0 + i % bxn;
-      red_row<F>(tl + (size_t)table_row(e, l, (uint32_t)vx, (uint32_t)vy) * F, v);
+      red_row<F, VEC>(tl + (size_t)table_row(e, l, (uint32_t)vx, (uint32_t)vy) * F, v);
     }
   }
 }
@@ -815,16 +817,20 @@ int table_grad(const Enc& e, const float* dX, long long sl, int si, int W, int H
   const TgPlan p = tg_plan(e, W, H, n0, count);
   const unsigned grid = (unsigned)p.pre[e.L];
   const size_t smem = (kTgSmem + 2 * kTgMaxRows) * sizeof(float);
+  const bool vec = (uintptr_t)dtable % (e.F == 2 ? 8 : 16) == 0;
+#define VS_TG(F, VEC) \
+  k_table_grad<F, VEC><<<grid, kTgThreads, smem, st>>>(e, p, dX, sl, si, W, H, n0, count, dtable)
   switch (e.F) {
-    case 1: k_table_grad<1><<<grid, kTgThreads, smem, st>>>(e, p, dX, sl, si, W, H, n0, count, dtable); break;
-    case 2: k_table_grad<2><<<grid, kTgThreads, smem, st>>>(e, p, dX, sl, si, W, H, n0, count, dtable); break;
-    case 3: k_table_grad<3><<<grid, kTgThreads, smem, st>>>(e, p, dX, sl, si, W, H, n0, count, dtable); break;
-    case 4: k_table_grad<4><<<grid, kTgThreads, smem, st>>>(e, p, dX, sl, si, W, H, n0, count, dtable); break;
-    case 5: k_table_grad<5><<<grid, kTgThreads, smem, st>>>(e, p, dX, sl, si, W, H, n0, count, dtable); break;
-    case 6: k_table_grad<6><<<grid, kTgThreads, smem, st>>>(e, p, dX, sl, si, W, H, n0, count, dtable); break;
-    case 7: k_table_grad<7><<<grid, kTgThreads, smem, st>>>(e, p, dX, sl, si, W, H, n0, count, dtable); break;
-    default: k_table_grad<8><<<grid, kTgThreads, smem, st>>>(e, p, dX, sl, si, W, H, n0, count, dtable); break;
+    case 1: VS_TG(1, false); break;
+    case 2: vec ? VS_TG(2, true) : VS_TG(2, false); break;
+    case 3: VS_TG(3, false); break;
+    case 4: vec ? VS_TG(4, true) : VS_TG(4, false); break;
+    case 5: VS_TG(5, false); break;
+    case 6: VS_TG(6, false); break;
+    case 7: VS_TG(7, false); break;
+    default: vec ? VS_TG(8, true) : VS_TG(8, false);
   }
+#undef VS_TG
   return (int)cudaGetLastError();
 }
 
@@ -840,13 +846,18 @@ int chunk_forward(const vs_ntex_config& c, const Enc& e, const Views& P, int W, 
   return 0;
 }
 
+// The fused kernels load rows of two features as one value.  Parameters need
+// 4-byte alignment only; where the rows are off an 8-byte boundary the layers
+// run one by one, behind k_encode, which then loads the features apart.
+bool fused_table(const Enc& e) { return e.F != 2 || e.pairs; }
+
 // The fused tensor-core forward (TF32 mode) for networks of 64-wide hidden
 // layers with at most 64 encoding values and outputs; one persistent launch
 // over the whole texture.  Returns -1 when the shape is not covered.
 int fused_forward_tc(const vs_ntex_config& c, const Views& P, const Enc& e, int W, int H, void* texels, int dtype,
                      int pitch, int ch0, int* status, cudaStream_t st) {
   const int LF = c.levels * c.features;
-  if (!c.tensor_cores || c.hidden != kMlpH || LF > 64 || c.out_ch > 64) return -1;
+  if (!c.tensor_cores || c.hidden != kMlpH || LF > 64 || c.out_ch > 64 || !fused_table(e)) return -1;
   const int smem = mlp_fwd_smem(LF, c.out_ch);
   static bool configured = false;
   if (!configured) {
@@ -889,7 +900,7 @@ int launch_fwd_f32(const F32FwdArgs& a, const Enc& e, cudaStream_t st) {
 int fused_forward_f32(const vs_ntex_config& c, const Views& P, const Enc& e, int W, int H, void* texels, int dtype,
                       int pitch, int ch0, cudaStream_t st) {
   const int LF = c.levels * c.features;
-  if (c.tensor_cores || c.hidden > 64 || LF > 64 || c.out_ch > 64) return -1;
+  if (c.tensor_cores || c.hidden > 64 || LF > 64 || c.out_ch > 64 || !fused_table(e)) return -1;
   const int vec = pitch % 4 == 0 && ch0 % 4 == 0 && (uintptr_t)texels % (dtype == 1 ? 8 : 16) == 0;
   const F32FwdArgs a{P.table, P.W0, P.b0, P.W1, P.b1, P.W2, P.b2, texels, W, H, W * H, c.out_ch, c.hidden, LF, dtype,
                      pitch, ch0, vec};
@@ -918,7 +929,7 @@ int launch_bwd_f32(const F32BwdArgs& a, const Enc& e, cudaStream_t st) {
 int fused_backward_f32(const vs_ntex_config& c, const Views& P, float* const g[7], const Enc& e, int W, int H,
                        const float* grad, int pitch, int ch0, void* ws, cudaStream_t st) {
   const int LF = c.levels * c.features;
-  if (c.tensor_cores || c.hidden > 64 || LF > 64 || c.out_ch > kBwdCP) return -1;
+  if (c.tensor_cores || c.hidden > 64 || LF > 64 || c.out_ch > kBwdCP || !fused_table(e)) return -1;
   const int vec = pitch % 4 == 0 && ch0 % 4 == 0 && (uintptr_t)grad % 16 == 0;
   // equal chunks of texels whose dX fits the workspace (sized for every
   // activation of kNtexChunk texels)
@@ -944,7 +955,7 @@ int forward(const vs_ntex_config& c, const float* params, int W, int H, void* te
   const float* v[7];
   views(c, params, v);
   const Views P{v[0], v[1], v[2], v[3], v[4], v[5], v[6]};
-  const Enc e = make_enc(c);
+  const Enc e = make_enc(c, P.table);
   const int N = W * H;
   {
     int r = fused_forward_f32(c, P, e, W, H, texels, dtype, pitch, ch0, st);
@@ -970,7 +981,8 @@ int forward(const vs_ntex_config& c, const float* params, int W, int H, void* te
 int fused_backward_tc(const vs_ntex_config& c, const Views& P, float* const g[7], const Enc& e, int W, int H,
                       const float* grad, int pitch, int ch0, void* ws, cudaStream_t st) {
   const int LF = c.levels * c.features;
-  if (!c.tensor_cores || c.hidden != kMlpH || LF > 32 || c.out_ch > 32 || 16 % c.features != 0) return -1;
+  if (!c.tensor_cores || c.hidden != kMlpH || LF > 32 || c.out_ch > 32 || 16 % c.features != 0 || !fused_table(e))
+    return -1;
   const int smem = mlp_bwd_smem(LF, c.out_ch);
   if (smem > 227 * 1024) return -1;
   static bool configured = false;
@@ -1008,7 +1020,7 @@ int backward(const vs_ntex_config& c, const float* params, int W, int H, const f
   const Views P{v[0], v[1], v[2], v[3], v[4], v[5], v[6]};
   float* g[7];
   views(c, grads, g);
-  const Enc e = make_enc(c);
+  const Enc e = make_enc(c, P.table);
   {
     int r = fused_backward_f32(c, P, g, e, W, H, grad_texels, pitch, ch0, ws, st);
     if (r >= 0) return r;

@@ -221,8 +221,8 @@ vs_status vs_workspace_size(vs_ctx* ctx, const vs_object* const* objs, const vs_
  *             shell's nearest front-facing hit, -1 = miss; may be NULL.
  *             The only state vs_render_backward needs.
  *   workspace device, >= vs_workspace_size(obj, cam, 1), 256-byte aligned
- * Launches, in order: the item-table upload, clear + vertex setup, raster,
- * shade + composite. */
+ * Launches, in order: clear + vertex setup (which carries the item table in
+ * its parameters), raster, shade + composite. */
 vs_status vs_render(vs_ctx* ctx, const vs_object* obj, const vs_camera* cam, const float* bg,
                     float* out_rgba, int32_t* hits, void* workspace, size_t ws_bytes,
                     uint32_t flags, vs_stream_t stream);
@@ -310,12 +310,17 @@ vs_status vs_render_batch(vs_ctx* ctx, const vs_batch_item* items, int32_t n, co
 
 /* Launch shape of vs_render_batch.  The paper's renderer has no such knobs
  * (a GL pipeline bins and tiles in fixed function); these are the work-unit
- * ("tile") sizes of the persistent kernel and its grid. */
+ * ("tile") sizes of the persistent kernel and its grid.  The sizes are upper
+ * bounds.  A batch cuts its raster units where warps would find none or a
+ * shell's triangles are large in the image (down to 8 triangles; one item
+ * alone down to one, shared by up to 64 units), and the shading units of its
+ * last item while warps would find none (down to 64 pixels).  Where these cuts
+ * decide, several tunings are the same launch. */
 typedef struct {
-  int32_t raster_tris;    /* triangles per raster work unit: a power of two in
-                             [32, 2048]                                       */
-  int32_t shade_pixels;   /* pixels per shading work unit: a power of two in
-                             [32, 4096]                                       */
+  int32_t raster_tris;    /* most triangles per raster work unit: a power of
+                             two in [32, 2048]                                */
+  int32_t shade_pixels;   /* most pixels per shading work unit: a power of two
+                             in [32, 4096]                                    */
   int32_t blocks_per_sm;  /* persistent blocks per SM (blocks of 160
                              threads with do_backward, else 224); 0 = the
                              occupancy maximum, else 1 .. that maximum
@@ -406,7 +411,8 @@ typedef struct {
 vs_status vs_ntex_layout(const vs_ntex_config* cfg, int64_t offsets[7], int64_t* total);
 
 /* Workspace bytes for vs_ntex_forward / vs_ntex_backward on a tex_w x tex_h
- * texture (activations of up to 2^18 texels at a time).  Host only.  Its
+ * texture (room for every activation of up to 2^18 texels at a time; kernels
+ * that keep activations on the chip use it for more texels).  Host only.  Its
  * first 4 bytes are a status word: zero the workspace once; with
  * tensor_cores = 1 a bounded wait that ran out writes 1 there (the layer's
  * outputs are then zero) and the call still returns. */
@@ -414,9 +420,12 @@ vs_status vs_ntex_workspace_size(const vs_ntex_config* cfg, int32_t tex_w, int32
 
 /* Evaluates the network at every texel centre and writes channels
  * [ch0, ch0 + C) of texels [tex_h, tex_w, pitch] (dtype 0 = float32,
- * 1 = float16, the renderer's SH storage).  FP32 arithmetic: the layers as
- * hand-written FP32 GEMMs with bias and ReLU fused, or on the tensor cores
- * in TF32 when cfg->tensor_cores = 1.
+ * 1 = float16, the renderer's SH storage).  FP32 arithmetic: encoding and
+ * layers in one kernel up to 64 encoding values, hidden units and outputs (32
+ * outputs for the adjoint), else a hand-written GEMM per layer; or the layers
+ * on the tensor cores in TF32 when cfg->tensor_cores = 1.  params (and grads)
+ * are 4-byte aligned; off an 8-byte boundary two features per level take the
+ * GEMMs.
  * Errors: VS_ERR_INVALID_ARG (config, sizes, ch0 + C > pitch, NULL),
  * VS_ERR_WORKSPACE, VS_ERR_CUDA. */
 vs_status vs_ntex_forward(vs_ctx* ctx, const vs_ntex_config* cfg, const float* params, int32_t tex_w, int32_t tex_h,
@@ -476,7 +485,7 @@ typedef struct {
   uint64_t tris_culled_back; /* back-facing or zero-area                       */
   uint64_t tris_culled_near; /* every vertex nearer than znear                */
   uint64_t tris_culled_guard;/* a vertex beyond +-32768 px                    */
-  uint64_t tris_large;       /* rasterized cooperatively by a whole block     */
+  uint64_t tris_large;       /* front-facing, box of more than 64 pixels      */
   uint64_t launches;         /* kernels enqueued by the calls (table uploads
                                 included), as declared by the host side      */
   uint64_t tris_clipped;     /* one or two vertices nearer than znear: clipped

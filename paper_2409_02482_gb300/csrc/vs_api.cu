@@ -248,10 +248,10 @@ struct UnitShape {
 // Setup units of an item of `verts` vertices and `words` visibility words to
 // clear: the largest size at which every warp asked for finds one of each
 // kind, but no fewer than 32 vertices (one per lane) and 512 words (8 stores
-// of 512 bytes).  At the largest size, 1024 vertices one after the other per
-// lane were the critical path of a single view: 25 us for the setup of an
-// 800^2 view of 7 x 200 k triangles, and as much for
-// that of a 256^2 view of 3 x 1.2 k, which takes 2.5 us in small units.
+// of 512 bytes).  At the largest size a lane takes 32 vertices one after the
+// other, which is the critical path of a single view: 25 us for the setup of
+// an 800^2 view of 7 x 200 k triangles, and as much for that of a 256^2 view
+// of 3 x 1.2 k, which takes 2.5 us in small units.
 void setup_shape(long long verts, long long words, const UnitShape& shape, int* uv, int* uw) {
   *uv = kSetupVerts;
   *uw = kClearWords;

@@ -41,7 +41,9 @@ constexpr int kRasterBlocks = 4;
 // / 161.2 / 164.1 us, 1080p baked frame 349 / 346 / 342 / 345; in the batch,
 // where views overlap, 32 views at 800^2 4.29 / 4.30 / 4.33 / 4.56 ms, fitting
 // step of 24 views 8.28 / 8.31 / 8.31 / 8.48, 4 views in 4K 10.09 / 10.50 /
-// 10.88 / 11.7.
+// 10.88 / 11.7.  Narrow images leave lanes idle at any width; 16 views of 1000
+// rows and 5 x 20 k triangles take 143 us at 1 pixel wide, 156 at 3, 202 at 7,
+// 296 at 20, 367 at 33 and 547 at 100.
 constexpr int kPlainTile = 8, kBatchTile = 32;
 constexpr int kMaxShells = VS_MAX_SHELLS;
 constexpr int kTriBits = 27;           // triangle index bits in a packed fragment
@@ -105,6 +107,10 @@ __host__ __device__ constexpr size_t block_smem_bytes(int K, bool bwd, int tc) {
 // 4 % slower).  The forward runs 7-warp blocks, 4 per SM: 28 warps at 72
 // registers (32 views at 800^2 4.30 ms, 4 in 4K 10.36 ms; 24 warps at 80
 // registers 4.43 / 10.45 ms, 32 at 64 4.47 / 10.58, 21 at 96 4.62 / 10.34).
+// 8 views at 800^2 in the other classes, 28 / 24 warps: SH0 906 / 887 us, SH1
+// 1027 / 1013, SH3 1599 / 1534, RGBA 899 / 880, baked degree 0 to 3 852 / 841,
+// 1115 / 1132, 1402 / 1383, 1773 / 1785, mixed formats 1187 / 1153, clipped
+// 2592 / 2448.
 #ifndef VS_PERS_BWD_WARPS
 #define VS_PERS_BWD_WARPS 5
 #endif
@@ -118,8 +124,7 @@ __host__ __device__ constexpr size_t pers_smem_bytes(int K, bool bwd, int tc) {
 }
 
 
-// Phases of one item.  Large triangles are rasterized by the whole block
-// inside the raster unit that met them.
+// Phases of one item.
 enum { PH_SETUP = 0, PH_RASTER = 1, PH_SHADE = 2, NPH = 3 };
 
 constexpr int kInvalidX = -2147483647 - 1;   // vertex marker: culled

@@ -45,10 +45,10 @@ __global__ void __launch_bounds__(kThreads) k_setup(char* ws, const __grid_const
 // Raster: resident blocks only, every warp strides over the item's units (of
 // 32 triangles, or fewer where the mesh is too small to give every warp
 // one: see vs_units.h).  What bounds it: latency of the dependent index and
-// vertex loads and of the walk.  One block per 256 triangles, each of its
-// warps adding its counts to the workspace header by itself, made 87 k
-// atomics on one cache line of an 800^2 view of 7 x 200 k triangles, and they
-// were the kernel's time; now a block adds its counts once.
+// vertex loads and of the walk.  A block adds its counts to the workspace
+// header once: additions by each warp of 256 triangles are 87 k atomics on one
+// cache line for an 800^2 view of 7 x 200 k triangles, and they are then the
+// kernel's time.
 template <bool FULL>
 __global__ void __launch_bounds__(kThreads, kRasterBlocks) k_raster(TableRef tb, int item) {
   __shared__ unsigned s_count[7];

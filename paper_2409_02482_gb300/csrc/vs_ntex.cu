@@ -7,15 +7,17 @@
 // gradients (vs_render_backward / the fused batch) back to the hash tables
 // and MLP parameters; vs_adam_step updates them.
 //
-// GB300 mapping.  FP32 layers (the default): per chunk of kNtexChunk texels
-// the encoding (a 4-corner gather per level, one thread per (texel, level)),
-// the three layers as hand-written GEMM kernels on the FP32 pipes with their
-// elementwise work fused in (bias and ReLU in the forward's epilogue, the
-// ReLU mask and the bias gradient's column sums in the adjoint's), so that
-// the activations (64 MB per layer at 2^18 texels) stay within L2 between
-// layers and in a bounded workspace.  TF32 layers (cfg.tensor_cores): one
-// fused persistent kernel each way, the layers on the tensor cores (tcgen05,
-// FP32 accumulators in tensor memory; vs_ntex_tc.cuh).  Both modes take the
+// GB300 mapping.  FP32 layers (the default): one fused kernel each way, the
+// activations in shared memory and every product an FP32 FMA
+// (vs_ntex_f32.cuh).  TF32 layers (cfg.tensor_cores): one fused persistent
+// kernel each way, the layers on the tensor cores (tcgen05, FP32 accumulators
+// in tensor memory; vs_ntex_tc.cuh).  Networks that the fused kernels do not
+// take run layer by layer, per chunk of kNtexChunk texels: the encoding (a
+// 4-corner gather per level, one thread per (texel, level)), then hand-written
+// GEMM kernels with the elementwise work fused in (bias and ReLU in the
+// forward's epilogue, the ReLU mask and the bias gradient's column sums in the
+// adjoint's), so that the activations (64 MB per layer at 2^18 texels) stay
+// within L2 between layers and in a bounded workspace.  All take the
 // encoding's adjoint in k_table_grad, by 2D tiles of texels (register runs
 // down columns, a shared vertex box per tile).
 
@@ -195,10 +197,13 @@ __global__ void __launch_bounds__(kThreads) k_encode(const __grid_constant__ Enc
 // atomics than the texels' corners), straight into the table.  A coarse
 // level thus takes a few atomics per tile instead of four per texel.
 // What bounds it: the latency of a column's loads (and, at the coarse levels,
-// of the shared atomics).  A column's texels were loaded one at a time, each
-// behind the lattice arithmetic of its row, the same in every thread; now the
-// rows' cells come from shared memory and four rows' loads are in flight
-// together (2^21 texels of 16 x 2 values: 310 -> 240 us; 268 MB of dX).
+// of the shared atomics).  So the lattice cells of the tile's rows, the same in
+// every thread, come from shared memory, and four rows' loads are in flight
+// together, against one row behind its own lattice arithmetic: 310 -> 240 us
+// for 2^21 texels of 16 x 2 values (268 MB of dX).  Other feature counts, the
+// whole TF32 adjoint at 1024^2: 16 x 1 1262 -> 1205 us, 12 x 3 6994 -> 6870,
+// 12 x 4 7406 -> 7178, 12 x 5 7790 -> 7544, 8 x 6 7622 -> 7452, 8 x 7 7914 ->
+// 7695, 8 x 8 8402 -> 8031.
 // Element (l, i, f) of dX (texel n0 + i) sits at dX[l sl + i si + f].
 constexpr int kTgThreads = 256;
 constexpr int kTgMaxRows = 128;  // rows of the tallest tile
@@ -882,7 +887,7 @@ int fused_forward_tc(const vs_ntex_config& c, const Views& P, const Enc& e, int 
 // values, padded with zeros to 32 or 64, and up to 64 outputs forward, 32
 // backward (the shared memory of a wider group would leave one per SM); other
 // shapes run the layer-by-layer kernels.  A 16 x 2 -> 64 -> 64 -> 27 network
-// at 2048^2: forward 1.59 ms fused, 5.44 ms layer by layer; adjoint 5.11 ms
+// at 2048^2: forward 1.59 ms fused, 5.44 ms layer by layer; adjoint 4.97 ms
 // against 17.9 ms.
 template <int HP, int LP, int CP>
 int launch_fwd_f32(const F32FwdArgs& a, const Enc& e, cudaStream_t st) {
